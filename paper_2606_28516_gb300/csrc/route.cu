@@ -15,7 +15,7 @@
 //   (64 columns) of a block, loaded as 16 TMA boxes of 8 rows x nkc K blocks (128-byte swizzle), so
 //   that every box reads nkc x 128 contiguous bytes of each of its rows (a box of 128 rows x 64
 //   columns, 128 bytes per row, kept DRAM 45 % busy); W_g sits in shared memory as the B operand (16
-//   rows, rows past E read as zero). One thread issues tcgen05.mma (M = 128, N = 16, K = 16, fp32
+//   rows, rows past E read as zero). One warp issues tcgen05.mma (M = 128, N = 16, K = 16, fp32
 //   accumulator in tensor memory, two accumulators); four epilogue warps, one per TMEM lane quarter,
 //   read their 32 rows' logits with tcgen05.ld, take the argmax per row (one row per lane, no
 //   shuffles) and the ranks by one ballot per expert, exchanging the four warps' counts through
@@ -117,13 +117,13 @@ __global__ void __launch_bounds__(RTC_THREADS, 1) route_tc_kernel(const __grid_c
     volatile int* abort_flag = &s_abort;
     const uint64_t lim = (uint64_t)a.wait_limit_ns;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const int E = a.E, nk = a.d / RTC_BK, nkc = lay.nkc, nh = nk / nkc;
     const uint32_t stage_bytes = (uint32_t)lay.stage_bytes, box_bytes = (uint32_t)nkc * RTC_BOX_ROWS * RTC_BK * 2;
     const int64_t row0 = (int64_t)blockIdx.x * A.chunk;
     const int nrows = (int)max((int64_t)0, min((int64_t)A.chunk, a.T - row0));
     const int nblk = (nrows + RTC_BM - 1) / RTC_BM;
-    const bool producer = warp == 4 && lane == 0, issuer = warp == 5 && lane == 0;
+    const bool producer = warp == 4, issuer = warp == 5;  // whole warps, one elected lane issues
 
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(RTC_THREADS, 1) route_tc_kernel(const __grid_c
     tc_fence_after();
     // W_g (a weight, not written by the previous kernel) is requested before the launch-overlap wait
     if (producer && nblk > 0) {
-        mbar_arrive_expect_tx(wbar, (uint32_t)(nk * RTC_WBOX_BYTES));
+        mbar_arrive_expect_tx_warp(wbar, (uint32_t)(nk * RTC_WBOX_BYTES));
         for (int kc = 0; kc < nk; ++kc) tma_load_2d(w_u32 + kc * RTC_WBOX_BYTES, &A.tmW, kc * RTC_BK, 0, wbar);
     }
     pdl_wait();  // from here on the previous kernel's results (x) are read and outputs written
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(RTC_THREADS, 1) route_tc_kernel(const __grid_c
         s_g[tid] = (a.ln_stats && tid < E) ? a.ln_wsum[tid] : 0.f;
     }
     __syncthreads();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
 
     if (producer) {
         // stage k = K blocks [h nkc, +nkc) of block j, with j = k / nh and h = k % nh; ring slot k % S
@@ -170,37 +170,37 @@ __global__ void __launch_bounds__(RTC_THREADS, 1) route_tc_kernel(const __grid_c
             const uint32_t bytes = (uint32_t)nbox * box_bytes;
             for (int h = 0; h < nh; ++h, ++k) {
                 const int s = k % S;
-                if (!mbar_wait(empty_bar(s), ((k / S) & 1) ^ 1, abort_flag, a.status, lim)) {
+                if (!mbar_wait_warp(empty_bar(s), ((k / S) & 1) ^ 1, abort_flag, a.status, lim)) {
                     ok = false;
                     break;
                 }
                 if (k == a.debug_skip && blockIdx.x == 0) continue;  // fault injection: withhold a stage
                 const uint32_t dst = ring_u32 + (uint32_t)s * stage_bytes;
-                mbar_arrive_expect_tx(full_bar(s), bytes);
+                mbar_arrive_expect_tx_warp(full_bar(s), bytes);
                 for (int b = 0; b < nbox; ++b)
                     tma_load_3d(dst + (uint32_t)b * box_bytes, &A.tmX, 0, r + b * RTC_BOX_ROWS, h * nkc, full_bar(s));
             }
         }
         if (!ok)  // gave up: let the copies in flight land before the CTA moves on
             for (int j = max(0, k - S); j < k; ++j)
-                mbar_wait(full_bar(j % S), (j / S) & 1, nullptr, a.status, 10000000ull);
-        if (nblk > 0) mbar_wait(wbar, 0, nullptr, a.status, 10000000ull);  // W_g's boxes have landed too
+                mbar_wait_warp(full_bar(j % S), (j / S) & 1, nullptr, a.status, 10000000ull);
+        if (nblk > 0) mbar_wait_warp(wbar, 0, nullptr, a.status, 10000000ull);  // W_g's boxes have landed too
     } else if (issuer) {
         const uint32_t idesc = idesc_bf16_f32(RTC_BM, 16);
         // a K block's descriptor is the ring base's plus the byte offset / 16 (addresses stay below
         // 256 KB): 8-row atoms nkc KB apart in x's stages, 1 KB apart in W_g's boxes
         const uint64_t dA0 = sdesc_kmajor_sw128_sbo(ring_u32, (uint32_t)nkc * 1024u);
         const uint64_t dW0 = sdesc_kmajor_sw128(w_u32);
-        bool ok = nblk == 0 || mbar_wait(wbar, 0, abort_flag, a.status, lim);
+        bool ok = nblk == 0 || mbar_wait_warp(wbar, 0, abort_flag, a.status, lim);
         int k = 0;
         for (int j = 0; j < nblk && ok; ++j) {
             const int acc = j & 1;
-            if (!mbar_wait(tempty_bar(acc), ((j >> 1) & 1) ^ 1, abort_flag, a.status, lim)) break;
+            if (!mbar_wait_warp(tempty_bar(acc), ((j >> 1) & 1) ^ 1, abort_flag, a.status, lim)) break;
             tc_fence_after();
             const uint32_t dtm = tmem + (uint32_t)acc * 16;
             for (int h = 0; h < nh; ++h, ++k) {
                 const int s = k % S;
-                if (!mbar_wait(full_bar(s), (k / S) & 1, abort_flag, a.status, lim)) {
+                if (!mbar_wait_warp(full_bar(s), (k / S) & 1, abort_flag, a.status, lim)) {
                     ok = false;
                     break;
                 }
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(RTC_THREADS, 1) route_tc_kernel(const __grid_c
             umma_commit(tfull_bar(acc));
         }
         umma_commit(drain_bar);  // every MMA issued has completed before tensor memory is released
-        mbar_wait(drain_bar, 0, nullptr, a.status, 10000000ull);
+        mbar_wait_warp(drain_bar, 0, nullptr, a.status, 10000000ull);
     } else if (warp < 4) {
         // epilogue: warp q reads TMEM lanes [32 q, +32) = rows 32 q .. 32 q + 31 of each block. Every
         // warp runs all nblk iterations (a wait that gave up only skips the work), so the named

@@ -7,8 +7,8 @@
 //              column half w / 4), bias+GELU / column scale / plain, round to bf16, stage through
 //              shared memory, coalesced 16-byte stores; rows may be scattered (out[perm[slot]],
 //              Algorithm 3 step 6);
-//   warp 8     TMEM allocation and the single thread that issues tcgen05.mma (M=128, N=BN,
-//              K=16 per instruction) and tcgen05.commit;
+//   warp 8     TMEM allocation; issues tcgen05.mma (M=128, N=BN, K=16 per instruction) and
+//              tcgen05.commit by one elected lane, the whole warp in step;
 //   warp 9     TMA producer (dense / grouped modes): 128-byte-swizzled A and B tiles;
 //   warps 10-13 gather producers (gather mode): the A rows of fc1 are tokens picked by the routing
 //              permutation, so they are copied row by row with 16-byte cp.async straight into the
@@ -111,9 +111,10 @@ __device__ __forceinline__ float tf32_rna(float x) {  // x rounded to TF32 (low 
 __device__ __forceinline__ void umma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                           uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     int* s_prefix = reinterpret_cast<int*>(tmem_slot + 4);  // [CM_MAX_E + 1]
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform((int)threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t bar0 = smem_u32(bars);
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto empty_bar = [&](int s) { return bar0 + 8u * (C::STAGES + s); };
@@ -275,35 +276,37 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
         }
         __syncthreads();
     }
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
 
     int m_tiles;
     if (MODE == TC_GROUPED)
         m_tiles = s_prefix[a.E];
     else
         m_tiles = (int)((a.M + TC_BM - 1) / TC_BM);
-    const int num_tiles = m_tiles * n_tiles;
+    const int num_tiles = warp_uniform(m_tiles * n_tiles);
 
     if (MODE != TC_GATHER && warp == TC_WARP_TMA) {
-        // ------------------------------------------------ TMA producer
-        if (lane == 0) {
+        // ------------------------------------------------ TMA producer (the whole warp)
+        {
             int stage = 0;
             uint32_t ph = 0;
             uint32_t issued = 0;  // bit s: stage s has a load in flight or done
             uint32_t par = 0;     // bit s: parity of stage s's last load
             bool ok = true;
             for (int unit = blockIdx.x; unit < num_tiles * ksp && ok; unit += gridDim.x) {
-                const TileInfo t = decode_tile(a, unit / ksp, n_tiles, s_prefix, BN);
+                TileInfo t = decode_tile(a, unit / ksp, n_tiles, s_prefix, BN);
+                t.e = warp_uniform(t.e);
+                t.m0 = warp_uniform(t.m0);
                 int klo, khi;  // the dense path's group (class tokens): the z x W2 segment alone
                 k_range(t, unit % ksp, klo, khi);
                 for (int kb = klo; kb < khi; ++kb) {
-                    if (!mbar_wait(empty_bar(stage), ph ^ 1, abort_flag, a.status, lim)) {
+                    if (!mbar_wait_warp(empty_bar(stage), ph ^ 1, abort_flag, a.status, lim)) {
                         ok = false;
                         break;
                     }
                     const uint32_t sA = smem_u32(sm + stage * C::STAGE_BYTES);
                     const uint32_t sB = sA + C::A_BYTES;
-                    mbar_arrive_expect_tx(full_bar(stage), C::HALF_BYTES);
+                    mbar_arrive_expect_tx_warp(full_bar(stage), C::HALF_BYTES);
                     if (kb < nk0) {
                         tma_load_2d(sA, &a.tmA0, kb * KE, (int)t.m0, full_bar(stage));
                         tma_load_2d(sB, &a.tmB0, kb * KE, t.n0, full_bar(stage));
@@ -322,7 +325,7 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
             }
             if (!ok) {  // let every copy in flight land before the CTA retires
                 for (int s = 0; s < C::STAGES; ++s)
-                    if (issued & (1u << s)) mbar_wait(full_bar(s), (par >> s) & 1, nullptr, a.status, 10000000ull);
+                    if (issued & (1u << s)) mbar_wait_warp(full_bar(s), (par >> s) & 1, nullptr, a.status, 10000000ull);
             }
         }
     } else if (TF32 && warp >= TC_WARP_GATHER) {
@@ -379,14 +382,14 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
                 if ((uint64_t)src[i] >= (uint64_t)a.M) src[i] = -1;  // only a launch that gave up leaves such rows
             }
             for (int kb = 0; kb < nkb; ++kb) {
-                if (!mbar_wait(empty_bar(stage), ph ^ 1, abort_flag, a.status, lim)) {
+                if (!mbar_wait_warp(empty_bar(stage), ph ^ 1, abort_flag, a.status, lim)) {
                     ok = false;
                     break;
                 }
                 const uint32_t sA = smem_u32(sm + stage * C::STAGE_BYTES);
                 const uint32_t sB = sA + C::A_BYTES;
-                if (pt == 0) {
-                    mbar_arrive_expect_tx(full_bar(stage), C::B_BYTES);
+                if (pt < 32) {  // warp-uniform; one elected lane issues
+                    mbar_arrive_expect_tx_warp(full_bar(stage), C::B_BYTES);
                     tma_load_2d(sB, &a.tmB0, kb * TC_BK, t.n0, full_bar(stage));
                 }
 #pragma unroll
@@ -406,47 +409,60 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
         }
         cp_async_wait<0>();
     } else if (warp == TC_WARP_MMA) {
-        // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        // ------------------------------------------------ MMA issuer (the whole warp)
+        {
             const uint32_t idesc = TF32 ? idesc_tf32_f32(TC_BM, BN) : idesc_bf16_f32(TC_BM, BN);
+            // stage s's descriptors are the stage-0 ones plus the byte offset / 16 in the start address
+            // field (every shared address here is below 256 KB, so the field never carries)
+            const uint64_t d0 = sdesc_kmajor_sw128(smem_u32(sm));
             int stage = 0;
             uint32_t ph = 0;
             int acc = 0;
             uint32_t aph = 0;
             bool ok = true;
             for (int unit = blockIdx.x; unit < num_tiles * ksp && ok; unit += gridDim.x) {
-                if (!mbar_wait(tempty_bar(acc), aph ^ 1, abort_flag, a.status, lim)) break;
+                if (!mbar_wait_warp(tempty_bar(acc), aph ^ 1, abort_flag, a.status, lim)) break;
                 tc_fence_after();
                 const uint32_t dtm = tmem_base + acc * BN;
                 int kb0, khi;
                 k_range(decode_tile(a, unit / ksp, n_tiles, s_prefix, BN), unit % ksp, kb0, khi);
+                kb0 = warp_uniform(kb0);
+                khi = warp_uniform(khi);
                 for (int kb = kb0; kb < khi; ++kb) {
                     // fp32: the stage once split (its bytes landed before the split warps read them)
-                    if (!mbar_wait(TF32 ? split_bar(stage) : full_bar(stage), ph, abort_flag, a.status, lim)) {
+                    if (!mbar_wait_warp(TF32 ? split_bar(stage) : full_bar(stage), ph, abort_flag, a.status, lim)) {
                         ok = false;
                         break;
                     }
                     if (MODE == TC_GATHER || TF32) fence_proxy_async_smem();
                     tc_fence_after();
-                    const uint32_t sA = smem_u32(sm + stage * C::STAGE_BYTES);
-                    const uint32_t sB = sA + C::A_BYTES;
+                    const uint64_t da = d0 + (uint64_t)((stage * C::STAGE_BYTES) >> 4);
+                    const uint64_t db = da + (uint64_t)(C::A_BYTES >> 4);
                     const int kvalid = kb < nk0 ? min(KE, a.K0 - kb * KE) : min(KE, a.K1 - (kb - nk0) * KE);
                     if constexpr (TF32) {
-                        // K = 8 per MMA; columns past K were filled with zeros by the TMA
-                        const int steps = (kvalid + 7) >> 3;
-                        for (int k = 0; k < steps; ++k) {
-                            const uint64_t ah = sdesc_kmajor_sw128(sA + k * 32), bh = sdesc_kmajor_sw128(sB + k * 32);
-                            const uint64_t al = sdesc_kmajor_sw128(sA + C::HALF_BYTES + k * 32);
-                            const uint64_t bl = sdesc_kmajor_sw128(sB + C::HALF_BYTES + k * 32);
+                        // K = 8 per MMA (32 bytes = 2 descriptor units); columns past K were filled with
+                        // zeros by the TMA
+                        constexpr uint64_t lo = C::HALF_BYTES >> 4;  // the remainders' offset
+                        auto step = [&](int k) {
+                            const uint64_t ah = da + 2 * k, bh = db + 2 * k;
                             umma_tf32(dtm, ah, bh, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-                            umma_tf32(dtm, ah, bl, idesc, 1u);
-                            umma_tf32(dtm, al, bh, idesc, 1u);
+                            umma_tf32(dtm, ah, bh + lo, idesc, 1u);
+                            umma_tf32(dtm, ah + lo, bh, idesc, 1u);
+                        };
+                        if (kvalid == KE) {
+#pragma unroll
+                            for (int k = 0; k < KE / 8; ++k) step(k);
+                        } else {
+                            for (int k = 0; k < ((kvalid + 7) >> 3); ++k) step(k);
                         }
                     } else {
-                        const int steps = kvalid >> 4;
-                        for (int k = 0; k < steps; ++k)
-                            umma_bf16(dtm, sdesc_kmajor_sw128(sA + k * 32), sdesc_kmajor_sw128(sB + k * 32),
-                                      idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+                        auto step = [&](int k) { umma_bf16(dtm, da + 2 * k, db + 2 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u); };
+                        if (kvalid == KE) {
+#pragma unroll
+                            for (int k = 0; k < KE / 16; ++k) step(k);
+                        } else {
+                            for (int k = 0; k < (kvalid >> 4); ++k) step(k);
+                        }
                     }
                     umma_commit(empty_bar(stage));
                     if (++stage == C::STAGES) {
@@ -460,7 +476,7 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
                 if (acc == 0) aph ^= 1;
             }
             umma_commit(drain_bar);  // every MMA issued above has completed once this fires
-            mbar_wait(drain_bar, 0, nullptr, a.status, 10000000ull);
+            mbar_wait_warp(drain_bar, 0, nullptr, a.status, 10000000ull);
         }
         __syncwarp();
     } else if (warp < TC_NUM_EPI) {

@@ -1,7 +1,7 @@
 // 2-SM bf16 GEMMs of the CLEAR-MoE FFN (tcgen05 cta_group::2, sm_103a).
 //
 // A cluster of two CTAs (one per SM of a pair) computes a 256 x 256 tile: CTA r loads A rows
-// [m0 + 128 r, +128) and B rows [n0 + 128 r, +128) into its own shared memory, and one thread of
+// [m0 + 128 r, +128) and B rows [n0 + 128 r, +128) into its own shared memory, and one warp of
 // the even CTA issues tcgen05.mma.cta_group::2 (M = 256, N = 256, K = 16), which reads A split by M
 // and B split by N across the two CTAs and leaves rows [128 r, +128) of the accumulator in CTA r's
 // tensor memory. Each SM thus holds half of the B tile: a k-block costs it 32 KB of operands for
@@ -70,16 +70,20 @@ __device__ __forceinline__ void cluster_sync() {
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int32_t c0, int32_t c1,
                                                  uint32_t bar_cluster) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2"
+        " [%0], [%1, {%2, %3}], [%4];\n\t}" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar_cluster)
         : "memory");
 }
 __device__ __forceinline__ void tma_load_2d_pair_hint(uint32_t dst, const CUtensorMap* map, int32_t c0, int32_t c1,
                                                       uint32_t bar_cluster, uint64_t policy) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2.L2::cache_hint"
-        " [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2.L2::cache_hint"
+        " [%0], [%1, {%2, %3}], [%4], %5;\n\t}" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar_cluster), "l"(policy)
         : "memory");
 }
@@ -101,17 +105,27 @@ __device__ __forceinline__ uint64_t l2_policy_evict_first() {
 __device__ __forceinline__ void umma2_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                            uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 __device__ __forceinline__ void umma2_commit_both(uint32_t bar) {  // arrive on bar in both CTAs
     asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(
             bar),
         "h"((unsigned short)3)
+        : "memory");
+}
+__device__ __forceinline__ void umma2_commit_one(uint32_t bar) {  // arrive on this CTA's bar
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
         : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
@@ -185,7 +199,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
     int* s_prefix = reinterpret_cast<int*>(tmem_slot + 4);  // [CM_MAX_E + 1]
 
     if (!a.pdl_trigger_late) pdl_launch_dependents();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform((int)threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
     const bool leader = rank == 0;
     const uint32_t bar0 = smem_u32(bars);
@@ -331,7 +345,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
         }
         __syncthreads();
     }
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
     uint32_t peer_base;
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(peer_base) : "r"(map_to_rank(smem_u32(tmem_slot), rank ^ 1)));
     const bool tmem_ok = peer_base == tmem_base;
@@ -343,24 +357,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
         m_pairs = s_prefix[a.E];
     else
         m_pairs = (int)((a.M + 2 * BM - 1) / (2 * BM));
-    const int num_units = tmem_ok ? m_pairs * units_per_pair<VAR>(n_tiles) : 0;
+    const int num_units = warp_uniform(tmem_ok ? m_pairs * units_per_pair<VAR>(n_tiles) : 0);
     const int cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;
 
     if (warp == WARP_TMA) {
         // ------------------------------------------------ producers (both CTAs)
-        // Lane 0 waits for free stages and issues the tile loads; with the z rows gathered by slot
-        // (a1_rows) every lane issues one four-row gather per stage (32 x 4 = the CTA's 128 rows),
-        // otherwise lane 0 runs alone.
+        // The whole warp waits for free stages, one elected lane issues the tile loads; with the z rows
+        // gathered by slot (a1_rows) every lane issues one four-row gather per stage (32 x 4 = the
+        // CTA's 128 rows).
         const uint32_t full_leader0 = map_to_rank(full_bar(0), 0);
         const uint64_t pol_a = l2_policy_evict_first();
         constexpr bool gather = VAR == TC2_GATHER;
         bool waited = a.pdl_wait_role != 2;  // role 2: wait before the first t-segment load
         int stage = 0;
         uint32_t ph = 0;
-        bool ok = gather || lane == 0;
+        bool ok = true;
         for (int u = cid; u < num_units && ok; u += ncl) {
-            const PairTile t = decode_pair<BN, VAR>(a, u, n_tiles, s_prefix);
-            const int am = (int)(t.m0 + (int64_t)rank * BM);
+            PairTile t = decode_pair<BN, VAR>(a, u, n_tiles, s_prefix);
+            t.e = warp_uniform(t.e);
+            const int am = warp_uniform((int)(t.m0 + (int64_t)rank * BM));
             // the router unit: CTA r supplies W_g rows [16 r, +16) of the 256 x 32 MMA
             const int bn = t.router ? (int)rank * 16 : t.n0 + (int)rank * BH;
             const uint32_t stage_tx = t.router ? 2u * (A_BYTES + C::FR_B_BYTES) : 2u * STAGE_BYTES;
@@ -376,17 +391,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                 }
             }
             for (int kb = 0; kb < nkb_t; ++kb) {
-                int w_ok = 1;
-                if (lane == 0) w_ok = mbar_wait(empty_bar(stage), ph ^ 1, abort_flag, a.status, lim);
-                if constexpr (gather) w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
-                if (!w_ok) {
+                if (!mbar_wait_warp(empty_bar(stage), ph ^ 1, abort_flag, a.status, lim)) {
                     ok = false;
                     break;
                 }
                 const uint32_t sA = smem_u32(sm + stage * STAGE_BYTES);
                 const uint32_t sB = sA + A_BYTES;
                 const uint32_t fb = full_leader0 + 8u * stage;  // the even CTA's full barrier
-                if (leader && lane == 0) mbar_arrive_expect_tx(full_bar(stage), stage_tx);
+                if (leader) mbar_arrive_expect_tx_warp(full_bar(stage), stage_tx);
                 const CUtensorMap* mA;
                 const CUtensorMap* mB;
                 int kk;
@@ -411,13 +423,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                 }
                 if (gathered) {
                     tma_gather4_pair(sA + 512u * lane, mA, kk, gr[0], gr[1], gr[2], gr[3], fb);
-                } else if (lane == 0) {
+                } else {
                     if (a.a_evict_first)
                         tma_load_2d_pair_hint(sA, mA, kk, am, fb, pol_a);
                     else
                         tma_load_2d_pair(sA, mA, kk, am, fb);
                 }
-                if (lane == 0) tma_load_2d_pair(sB, mB, kk, bn, fb);
+                tma_load_2d_pair(sB, mB, kk, bn, fb);
                 if (++stage == STAGES) {
                     stage = 0;
                     ph ^= 1;
@@ -425,8 +437,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
             }
         }
     } else if (warp == WARP_MMA) {
-        // ------------------------------------------------ MMA issuer (even CTA)
-        if (leader && lane == 0) {
+        // ------------------------------------------------ MMA issuer (even CTA, the whole warp)
+        if (leader) {
             const uint32_t idesc_t = idesc_bf16_f32(2 * BM, BN);
             const uint32_t idesc_r = idesc_bf16_f32(2 * BM, 32);  // the router unit: 256 x 32
             const int nup = units_per_pair<VAR>(n_tiles);
@@ -439,15 +451,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
             uint32_t aph = 0;
             bool ok = true;
             for (int u = cid; u < num_units && ok; u += ncl) {
-                if (!mbar_wait(tempty_bar(acc), aph ^ 1, abort_flag, a.status, lim)) break;
+                if (!mbar_wait_warp(tempty_bar(acc), aph ^ 1, abort_flag, a.status, lim)) break;
                 tc_fence_after();
                 const uint32_t dtm = tmem_base + acc * BN;
                 const uint32_t idesc = (VAR == TC2_ROUTER && u % nup == n_tiles) ? idesc_r : idesc_t;
                 int nkb_t = nkb;  // the dense path's group: the z x W2 segment alone
-                if (MODE == TC_GROUPED && a.dense_last && decode_pair<BN, VAR>(a, u, n_tiles, s_prefix).e == a.E - 1)
+                if (MODE == TC_GROUPED && a.dense_last && warp_uniform(decode_pair<BN, VAR>(a, u, n_tiles, s_prefix).e) == a.E - 1)
                     nkb_t = nk1;
                 for (int kb = 0; kb < nkb_t; ++kb) {
-                    if (!mbar_wait(full_bar(stage), ph, abort_flag, a.status, lim)) {
+                    if (!mbar_wait_warp(full_bar(stage), ph, abort_flag, a.status, lim)) {
                         ok = false;
                         break;
                     }
@@ -480,9 +492,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                     aph ^= 1;
                 }
             }
-            asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(drain_bar)
-                         : "memory");
-            mbar_wait(drain_bar, 0, nullptr, a.status, 10000000ull);
+            umma2_commit_one(drain_bar);
+            mbar_wait_warp(drain_bar, 0, nullptr, a.status, 10000000ull);
         }
         __syncwarp();
     } else if (warp < NUM_EPI) {

@@ -220,8 +220,8 @@ struct TcGemmArgs {
     int epi12;
     // 1-SM kernel, dense and grouped modes: fp32 operands (tensor maps from encode_tmap_f32) on the
     // TF32 tensor cores with three products per K step (hi hi + hi lo + lo hi, each fp32 operand split
-    // into a TF32 part and its remainder in shared memory); bias, out_bias and C are fp32 (c_f32
-    // set), GELU is gelu_erf; no LayerNorm fold
+    // into a TF32 part and its remainder, A's in tensor memory); bias, out_bias and C are fp32 (c_f32
+    // set), GELU is gelu_pair_f32; no LayerNorm fold
     int tf32;
     // fp32 (TF32) variant: each tile's K blocks split into ksplit ranges (> 1 when tiles alone leave
     // SMs idle), one unit each; a unit stores its fp32 partial tile in ws ([tiles x ksplit x 128 x BN]),

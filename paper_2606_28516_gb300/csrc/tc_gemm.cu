@@ -21,13 +21,22 @@
 // copies and MMAs, frees TMEM and returns.
 //
 // The fp32 variant (TF32 = true, dense and grouped modes) runs fp32 operands on the TF32 tensor
-// cores (kind::tf32, K = 8 per instruction, the same 128-byte rows and descriptors as bf16): a TMA
-// box of 32 fp32 per row lands where 64 bf16 would, then warps 10-13 split every value v of the
-// stage into h = v rounded to TF32 (written back in place) and its exact remainder l = v - h
-// (written to a second half of the stage at the same offset), and each K step issues three MMAs,
-// h_A h_B + h_A l_B + l_A h_B, into the fp32 accumulator. The dropped l_A l_B and the TF32 rounding of
-// the remainders leave a relative error near 2^-21 per product, so fp32 layers keep their accuracy
-// on the tensor cores (one TF32 product alone would be off by up to 2^-11).
+// cores (kind::tf32, K = 8 per instruction): a TMA box of 32 fp32 per row lands where 64 bf16 would,
+// then warps 10-13 split every value v of the stage into h = v rounded to TF32 and its exact remainder
+// l = v - h, and each K step issues three MMAs, h_A h_B + h_A l_B + l_A h_B, into the fp32 accumulator.
+// The dropped l_A l_B and the TF32 rounding of the remainders leave a relative error near 2^-21 per
+// product, so fp32 layers keep their accuracy on the tensor cores (one TF32 product alone would be off
+// by up to 2^-11).
+// What bounds it: shared-memory bandwidth. With both operands split in place a 128 x 64 stage moves
+// 24 KB in by TMA, 24 KB to the split warps, 48 KB back and 72 KB to the MMAs; so A's two parts go to
+// tensor memory instead (one row per lane, 32 columns each) and the MMAs read them there, and only B is
+// written back: 88 KB instead of 168 KB per stage, and more stages fit. Four split warps: eight
+// measured slower (115 against 112 us, the whole layer below), as they share the bandwidth. The output
+// rows and the K-split partials are stored with consecutive lanes on consecutive bytes (one row per
+// lane touched 32 rows with 16 bytes each), and GELU takes the branch-free form of common.cuh.
+// Measured (DeiT-T layer, whole forwards): T = 12,608: 125 us with both operands in shared memory, 112
+// with coalesced stores, 93 with A in tensor memory, 87.5 with the branch-free GELU; T = 788: 48.1 /
+// 42.5 / 38.8 / 37.1 us. Results differ from the first form's only through GELU.
 #include <cstdint>
 #include <mutex>
 
@@ -45,6 +54,10 @@ constexpr int TC_WARP_GATHER = 10;
 constexpr int TC_GATHER_THREADS = 128;
 constexpr int TC_THREADS_TMA = 32 * (TC_WARP_TMA + 1);
 constexpr int TC_THREADS_GATHER = 32 * TC_WARP_GATHER + TC_GATHER_THREADS;
+template <int MODE, bool TF32>
+constexpr int tc_threads() {
+    return TF32 || MODE == TC_GATHER ? TC_THREADS_GATHER : TC_THREADS_TMA;
+}
 
 // K elements per stage: 64 bf16 or 32 fp32, a 128-byte row either way
 template <bool TF32>
@@ -56,16 +69,19 @@ template <int BN, bool TF32 = false>
 struct TcCfg {
     static constexpr int A_BYTES = TC_BM * TC_BK * 2;
     static constexpr int B_BYTES = BN * TC_BK * 2;
-    // fp32: the stage's second half holds the remainders of its first, at the same offsets
-    static constexpr int HALF_BYTES = A_BYTES + B_BYTES;
-    static constexpr int STAGE_BYTES = TF32 ? 2 * HALF_BYTES : HALF_BYTES;
-    static constexpr int STAGES_RAW = (196 * 1024) / STAGE_BYTES;
-    static constexpr int STAGES = STAGES_RAW > 8 ? 8 : STAGES_RAW;
+    static constexpr int LOAD_BYTES = A_BYTES + B_BYTES;
+    // fp32: B's remainders follow B; A's two parts go to tensor memory, 64 columns per stage after the
+    // two accumulators
+    static constexpr int STAGE_BYTES = TF32 ? LOAD_BYTES + B_BYTES : LOAD_BYTES;
+    static constexpr int A_COLS = 2 * (TC_BK / 2);
+    static constexpr int STAGES_SMEM = (196 * 1024) / STAGE_BYTES;
+    static constexpr int STAGES_CAP = TF32 && (512 - 2 * BN) / A_COLS < 8 ? (512 - 2 * BN) / A_COLS : 8;
+    static constexpr int STAGES = STAGES_SMEM > STAGES_CAP ? STAGES_CAP : STAGES_SMEM;
     static constexpr int HALF = BN / 2;               // columns per epilogue warp
     static constexpr int CW = HALF < 32 ? HALF : 32;  // epilogue columns per TMEM load
     static constexpr int STG_ROW = CW * 2 + 16;       // staging row pitch (bytes)
     static constexpr int STG_BYTES = TC_NUM_EPI * 32 * STG_ROW;
-    static constexpr int TMEM_COLS = (2 * BN <= 32) ? 32 : (2 * BN <= 64) ? 64 : (2 * BN <= 128) ? 128
+    static constexpr int TMEM_COLS = TF32 ? 512 : (2 * BN <= 32) ? 32 : (2 * BN <= 64) ? 64 : (2 * BN <= 128) ? 128
                                      : (2 * BN <= 256) ? 256 : 512;
     // + (fp32) the split stages' barriers and the two of the K-split handshake
     static constexpr int NBARS = 2 * STAGES + 5 + (TF32 ? STAGES + 2 : 0);
@@ -102,20 +118,22 @@ __device__ __forceinline__ TileInfo decode_tile(const TcGemmArgs& a, int tile, i
     return t;
 }
 
-__device__ __forceinline__ float tf32_rna(float x) {  // x rounded to TF32 (low 13 bits zero)
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
+// x rounded to TF32 (low 13 bits zero), to nearest, ties away from zero, as cvt.rna.tf32.f32 does, by
+// integer arithmetic (the conversion runs at a quarter of its rate). A NaN may come out as another
+// value, whose exact remainder is then NaN: the sum of the three products still is.
+__device__ __forceinline__ float tf32_rna(float x) {
+    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
 }
 
-__device__ __forceinline__ void umma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate) {
+// D[tmem] (+)= A[tmem] * B[smem]^T, kind::tf32: A's row m in lane m, one 32-bit column per k.
+__device__ __forceinline__ void umma_tf32_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                             uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "elect.sync _|q, 0xffffffff;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
@@ -124,8 +142,55 @@ __host__ __device__ constexpr uint32_t idesc_tf32_f32(int M, int N) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// Four fp32 values + bias, then GELU or ReLU for fc1's epilogues.
+__device__ __forceinline__ void f32_bias_act(float* f, float4 b, int epi) {
+    float2 p0 = __fadd2_rn(make_float2(f[0], f[1]), make_float2(b.x, b.y));
+    float2 p1 = __fadd2_rn(make_float2(f[2], f[3]), make_float2(b.z, b.w));
+    if (epi == TC_EPI_BIAS_GELU) {
+        p0 = gelu_pair_f32(p0);
+        p1 = gelu_pair_f32(p1);
+    } else if (epi == TC_EPI_BIAS_RELU) {
+        p0 = make_float2(fmaxf(p0.x, 0.f), fmaxf(p0.y, 0.f));
+        p1 = make_float2(fmaxf(p1.x, 0.f), fmaxf(p1.y, 0.f));
+    }
+    f[0] = p0.x;
+    f[1] = p0.y;
+    f[2] = p1.x;
+    f[3] = p1.y;
+}
+
+// fp32 rows of a warp (lane = row, CW values each in f) to C through shared memory, half a warp's rows at
+// a time: 16-byte piece j of row rw at piece j ^ (rw & mask), then each store instruction writes
+// 512 contiguous-by-row bytes (CW x 4 bytes per row) where one row per lane would touch 32 rows with 16
+// bytes each. wstg: 16 x CW x 4 bytes of the warp's own.
+template <int CW>
+__device__ __forceinline__ void store_rows_f32(unsigned char* wstg, int lane, const float* f, int64_t orow, float* C,
+                                               int64_t ldc, int nb) {
+    constexpr int LPR = CW / 4;   // lanes (16-byte pieces) per row
+    constexpr int RPP = 32 / LPR; // rows per store instruction
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if ((lane >> 4) == h) {
+            const int rw = lane & 15;
+#pragma unroll
+            for (int j = 0; j < LPR; ++j)
+                *reinterpret_cast<float4*>(wstg + rw * (CW * 4) + ((j ^ (rw & (LPR - 1))) << 4)) =
+                    make_float4(f[4 * j], f[4 * j + 1], f[4 * j + 2], f[4 * j + 3]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int p = 0; p < 16; p += RPP) {
+            const int rw = p + lane / LPR;
+            const int64_t o = __shfl_sync(0xffffffffu, orow, 16 * h + (rw & 15));
+            const float4 v = *reinterpret_cast<const float4*>(wstg + (rw & 15) * (CW * 4) + (((lane % LPR) ^ (rw & (LPR - 1))) << 4));
+            if (o >= 0 && rw < 16) *reinterpret_cast<float4*>(C + o * ldc + nb + (lane % LPR) * 4) = v;
+        }
+        __syncwarp();
+    }
+}
+
 template <int BN, int MODE, bool TF32>
-__global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHER : TC_THREADS_TMA, 1)
+__global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
     tc_gemm_kernel(const __grid_constant__ TcGemmArgs a) {
     if (!a.pdl_trigger_late) pdl_launch_dependents();
     using C = TcCfg<BN, TF32>;
@@ -306,7 +371,7 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
                     }
                     const uint32_t sA = smem_u32(sm + stage * C::STAGE_BYTES);
                     const uint32_t sB = sA + C::A_BYTES;
-                    mbar_arrive_expect_tx_warp(full_bar(stage), C::HALF_BYTES);
+                    mbar_arrive_expect_tx_warp(full_bar(stage), C::LOAD_BYTES);
                     if (kb < nk0) {
                         tma_load_2d(sA, &a.tmA0, kb * KE, (int)t.m0, full_bar(stage));
                         tma_load_2d(sB, &a.tmB0, kb * KE, t.n0, full_bar(stage));
@@ -330,9 +395,12 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
         }
     } else if (TF32 && warp >= TC_WARP_GATHER) {
         // ------------------------------------------------ fp32: split each landed stage
-        // v -> h = TF32(v) in place, l = v - h (exact) in the stage's second half; the writes are
-        // made visible to the tensor cores' (async) proxy before the warp's arrival.
+        // v -> h = TF32(v) and l = v - h (exact). A's rows (one per lane of its tensor memory quarter) go
+        // to tensor memory, h in 32 columns and l in the next 32; B's parts stay in shared memory, h in
+        // place and l behind it. Both are made visible to the tensor cores before the warp's arrival.
         const int ct = threadIdx.x - TC_WARP_GATHER * 32;
+        const int row = (warp & 3) * 32 + lane;
+        const uint32_t a_tmem = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + 2 * BN;
         int stage = 0;
         uint32_t ph = 0;
         bool ok = true;
@@ -340,21 +408,40 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
             const TileInfo t = decode_tile(a, unit / ksp, n_tiles, s_prefix, BN);
             int klo, khi;
             k_range(t, unit % ksp, klo, khi);
+            klo = warp_uniform(klo);
+            khi = warp_uniform(khi);
             for (int kb = klo; kb < khi; ++kb) {
-                if (!mbar_wait(full_bar(stage), ph, abort_flag, a.status, lim)) {
+                if (!mbar_wait_warp(full_bar(stage), ph, abort_flag, a.status, lim)) {
                     ok = false;
                     break;
                 }
-                float4* hi = reinterpret_cast<float4*>(sm + stage * C::STAGE_BYTES);
-                float4* lo = reinterpret_cast<float4*>(sm + stage * C::STAGE_BYTES + C::HALF_BYTES);
-#pragma unroll 4
-                for (int i = ct; i < C::HALF_BYTES / 16; i += TC_GATHER_THREADS) {
-                    const float4 v = hi[i];
-                    const float4 h = make_float4(tf32_rna(v.x), tf32_rna(v.y), tf32_rna(v.z), tf32_rna(v.w));
-                    hi[i] = h;
-                    lo[i] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
+                const unsigned char* sA = sm + stage * C::STAGE_BYTES + row * 128;
+                uint32_t h[32], l[32];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {  // 16-byte piece j of a row lies at piece j ^ (row & 7)
+                    const float4 v = *reinterpret_cast<const float4*>(sA + ((j ^ (row & 7)) << 4));
+                    const float f[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float hv = tf32_rna(f[i]);
+                        h[4 * j + i] = __float_as_uint(hv);
+                        l[4 * j + i] = __float_as_uint(f[i] - hv);
+                    }
+                }
+                CM_TMEM_ST_X32(a_tmem + stage * C::A_COLS, h);
+                CM_TMEM_ST_X32(a_tmem + stage * C::A_COLS + 32, l);
+                float4* bh = reinterpret_cast<float4*>(sm + stage * C::STAGE_BYTES + C::A_BYTES);
+                float4* bl = bh + C::B_BYTES / 16;
+#pragma unroll
+                for (int i = ct; i < C::B_BYTES / 16; i += TC_GATHER_THREADS) {
+                    const float4 v = bh[i];
+                    const float4 hv = make_float4(tf32_rna(v.x), tf32_rna(v.y), tf32_rna(v.z), tf32_rna(v.w));
+                    bh[i] = hv;
+                    bl[i] = make_float4(v.x - hv.x, v.y - hv.y, v.z - hv.z, v.w - hv.w);
                 }
                 fence_proxy_async_smem();
+                tmem_wait_st();
+                tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(split_bar(stage));
                 if (++stage == C::STAGES) {
@@ -442,12 +529,14 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
                     if constexpr (TF32) {
                         // K = 8 per MMA (32 bytes = 2 descriptor units); columns past K were filled with
                         // zeros by the TMA
-                        constexpr uint64_t lo = C::HALF_BYTES >> 4;  // the remainders' offset
+                        constexpr uint64_t lo = C::B_BYTES >> 4;  // B's remainders' offset
+                        const uint32_t at = tmem_base + 2 * BN + stage * C::A_COLS;  // A's parts
                         auto step = [&](int k) {
-                            const uint64_t ah = da + 2 * k, bh = db + 2 * k;
-                            umma_tf32(dtm, ah, bh, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-                            umma_tf32(dtm, ah, bh + lo, idesc, 1u);
-                            umma_tf32(dtm, ah + lo, bh, idesc, 1u);
+                            const uint32_t ah = at + 8 * k;
+                            const uint64_t bh = db + 2 * k;
+                            umma_tf32_ts(dtm, ah, bh, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+                            umma_tf32_ts(dtm, ah, bh + lo, idesc, 1u);
+                            umma_tf32_ts(dtm, ah + 32, bh, idesc, 1u);
                         };
                         if (kvalid == KE) {
 #pragma unroll
@@ -538,10 +627,11 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
                 for (int j = 0; j < C::CW; ++j) f[j] = klo < khi ? __uint_as_float(v[j]) : 0.f;
                 if (TF32 && ksp > 1) {  // a K range's partial tile, finished by the tile's last unit below
                     if (r < t.rows) {
-                        float4* w4 = reinterpret_cast<float4*>(a.ws + ((int64_t)unit * TC_BM + r) * BN + c);
+                        // [unit][column / 4][row]: consecutive lanes (rows) store consecutive 16 bytes
+                        float4* w4 = reinterpret_cast<float4*>(a.ws) + ((int64_t)unit * (BN / 4) + c / 4) * TC_BM + r;
 #pragma unroll
                         for (int j4 = 0; j4 < C::CW / 4; ++j4)
-                            w4[j4] = make_float4(f[4 * j4], f[4 * j4 + 1], f[4 * j4 + 2], f[4 * j4 + 3]);
+                            w4[j4 * TC_BM] = make_float4(f[4 * j4], f[4 * j4 + 1], f[4 * j4 + 2], f[4 * j4 + 3]);
                     }
                     continue;
                 }
@@ -551,18 +641,13 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
                     for (int j = 0; j < C::CW; ++j) f[j] = ln.y * fmaf(-ln.x, __ldg(a.ln_colsum + nb + j), f[j]);
                 }
                 if (TF32 && (a.epi == TC_EPI_BIAS_GELU || a.epi == TC_EPI_BIAS_RELU || a.out_bias)) {
-                    // fp32 bias (b1, or fc2's b2), then GELU (CUDA's erff) or ReLU for fc1
+                    // fp32 bias (b1, or fc2's b2), then GELU or ReLU for fc1
                     const bool fc1 = a.epi == TC_EPI_BIAS_GELU || a.epi == TC_EPI_BIAS_RELU;
                     const float4* bp = reinterpret_cast<const float4*>(static_cast<const float*>(fc1 ? a.bias : a.out_bias) + nb);
 #pragma unroll
                     for (int j4 = 0; j4 < C::CW / 4; ++j4) {
                         const float4 b = __ldg(bp + j4);
-                        const float bb[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-                        for (int h = 0; h < 4; ++h) {
-                            const float v = f[4 * j4 + h] + bb[h];
-                            f[4 * j4 + h] = a.epi == TC_EPI_BIAS_GELU ? gelu_erf(v) : a.epi == TC_EPI_BIAS_RELU ? fmaxf(v, 0.f) : v;
-                        }
+                        f32_bias_act(f + 4 * j4, b, a.epi);
                     }
                 } else if (a.epi == TC_EPI_BIAS_GELU) {
                     const uint4* bp = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(a.bias) + nb);
@@ -617,13 +702,8 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
 #pragma unroll
                     for (int j = 0; j < C::CW; ++j) f[j] *= rsc;
                 }
-                if (a.c_f32) {  // fp32 output: each lane stores its row's values as computed
-                    if (orow >= 0) {
-                        float4* dstf = reinterpret_cast<float4*>(static_cast<float*>(a.C) + orow * a.ldc + nb);
-#pragma unroll
-                        for (int j4 = 0; j4 < C::CW / 4; ++j4)
-                            dstf[j4] = make_float4(f[4 * j4], f[4 * j4 + 1], f[4 * j4 + 2], f[4 * j4 + 3]);
-                    }
+                if (a.c_f32) {  // fp32 output: stored as computed
+                    store_rows_f32<C::CW>(wstg, lane, f, orow, static_cast<float*>(a.C), a.ldc, nb);
                     continue;
                 }
                 uint4* dst = reinterpret_cast<uint4*>(wstg + lane * C::STG_ROW);
@@ -665,18 +745,19 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
                 }
                 const bool done = mbar_wait(kdone_bar, kph, abort_flag, a.status, lim);
                 kph ^= 1;
-                if (done && *s_last && orow >= 0) {
+                // the warp agrees (a wait that gave up ends it for single lanes), so that its rows are stored together
+                if (__all_sync(0xffffffffu, done && *s_last)) {
                     __threadfence();
                     for (int c = c_lo; c < c_lo + C::HALF; c += C::CW) {
                         float f[C::CW];
 #pragma unroll
                         for (int j = 0; j < C::CW; ++j) f[j] = 0.f;
                         for (int sp = 0; sp < ksp; ++sp) {
-                            const float4* w4 =
-                                reinterpret_cast<const float4*>(a.ws + (((int64_t)tile * ksp + sp) * TC_BM + r) * BN + c);
+                            const float4* w4 = reinterpret_cast<const float4*>(a.ws) +
+                                               (((int64_t)tile * ksp + sp) * (BN / 4) + c / 4) * TC_BM + r;
 #pragma unroll
                             for (int j4 = 0; j4 < C::CW / 4; ++j4) {
-                                const float4 pv = __ldcg(w4 + j4);
+                                const float4 pv = __ldcg(w4 + j4 * TC_BM);
                                 f[4 * j4] += pv.x;
                                 f[4 * j4 + 1] += pv.y;
                                 f[4 * j4 + 2] += pv.z;
@@ -686,12 +767,10 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
                         const int nb = t.n0 + c;
                         if (a.epi == TC_EPI_BIAS_GELU || a.epi == TC_EPI_BIAS_RELU || a.out_bias) {
                             const bool fc1 = a.epi == TC_EPI_BIAS_GELU || a.epi == TC_EPI_BIAS_RELU;
-                            const float* bp = static_cast<const float*>(fc1 ? a.bias : a.out_bias) + nb;
+                            const float4* bp =
+                                reinterpret_cast<const float4*>(static_cast<const float*>(fc1 ? a.bias : a.out_bias) + nb);
 #pragma unroll
-                            for (int j = 0; j < C::CW; ++j) {
-                                const float v = f[j] + __ldg(bp + j);
-                                f[j] = a.epi == TC_EPI_BIAS_GELU ? gelu_erf(v) : a.epi == TC_EPI_BIAS_RELU ? fmaxf(v, 0.f) : v;
-                            }
+                            for (int j4 = 0; j4 < C::CW / 4; ++j4) f32_bias_act(f + 4 * j4, __ldg(bp + j4), a.epi);
                         } else if (a.epi == TC_EPI_SCALE) {
 #pragma unroll
                             for (int j = 0; j < C::CW; ++j) f[j] *= __ldg(a.scale + nb + j);
@@ -700,10 +779,7 @@ __global__ void __launch_bounds__((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHE
 #pragma unroll
                             for (int j = 0; j < C::CW; ++j) f[j] *= rsc;
                         }
-                        float4* dstf = reinterpret_cast<float4*>(static_cast<float*>(a.C) + orow * a.ldc + nb);
-#pragma unroll
-                        for (int j4 = 0; j4 < C::CW / 4; ++j4)
-                            dstf[j4] = make_float4(f[4 * j4], f[4 * j4 + 1], f[4 * j4 + 2], f[4 * j4 + 3]);
+                        store_rows_f32<C::CW>(wstg, lane, f, orow, static_cast<float*>(a.C), a.ldc, nb);
                     }
                 }
             }
@@ -770,7 +846,7 @@ static cudaError_t launch_one(const TcGemmArgs& a, int num_sms, cudaStream_t s) 
     if (grid <= 0) return cudaSuccess;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3((MODE == TC_GATHER || TF32) ? TC_THREADS_GATHER : TC_THREADS_TMA);
+    cfg.blockDim = dim3(tc_threads<MODE, TF32>());
     cfg.dynamicSmemBytes = C::SMEM;
     cfg.stream = s;
     cudaLaunchAttribute attr_pdl[1];

@@ -631,7 +631,7 @@ static int ffn_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W1,
     if ((rc = do_route(L, x, T, router, mlp, E, cls_stride, s, ln))) return rc;
     // bf16 with the 2-SM fc1, or fp32 on the tensor cores: the fc1 epilogue assigns the slots
     // itself (no finalize launch)
-    const int p1 = bf16 && H <= cm::TC2_BIAS_CAP ? cm::tc2_pick_bn(cm::TC_DENSE, H) : 0;
+    const int p1 = bf16 && H <= cm::TC2_BIAS_CAP ? cm::tc2_fc1_bn(T, H, d, true, L->num_sms) : 0;
     const bool f32_tc = !bf16 && !ln && f32_tc_ok(d, H, r, factored);
     const bool fused = (p1 || f32_tc) && L->rt_grid <= 256 && L->rt_grid * E <= cm::TC2_TAB_CAP;
     if (!fused && (rc = do_finalize(L, s))) return rc;
@@ -737,6 +737,7 @@ static int ffn_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W1,
             return CLEARMOE_ECUDA;
         if (ln && (rc = ln_fc1_aug(L, g, T, p1 / 2))) return rc;
         g.mode = cm::TC_DENSE;
+        g.bn = p1;
         if (fused) {  // slots from the routing's per-range counts and ranks; writes perm, counts, offsets
             g.rt_info = L->tinfo;
             g.rt_counts = L->cta_counts;
@@ -794,8 +795,9 @@ static int ffn_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W1,
     g3.status = L->status;
     g3.wait_limit_ns = L->wait_limit_ns;
     // The 2-SM kernel loads half of each pair tile's B rows per CTA: boxes of p3 / 2 rows.
-    const int p3 = cm::tc2_pick_bn(cm::TC_GROUPED, d);
+    const int p3 = cm::tc2_grouped_bn(T, d, G, factored ? (T - n_cls + 255) / 256 : 0, L->num_sms);
     const int box3 = p3 ? p3 / 2 : bn3;
+    g3.bn = p3;
     if ((factored && (encode_tmap_bf16(&g3.tmA0, L->t, T, r, 128) || encode_tmap_bf16(&g3.tmB0, U_r, d, r, box3))) ||
         (materialized &&
          (encode_tmap_bf16(&g3.tmA0, L->z, T, H, 128) || encode_tmap_bf16(&g3.tmB0, W_sh, d, H, box3))) ||
@@ -969,8 +971,8 @@ int clearmoe_ffn_forward_scaled(clearmoe_layer* L, const void* x, int64_t T, con
         g.ldc = d;
         rc = launch_simt(L, g, s);
     } else {
-        const int p1 = H <= cm::TC2_BIAS_CAP ? cm::tc2_pick_bn(cm::TC_DENSE, H) : 0;
-        const int p2 = cm::tc2_pick_bn(cm::TC_DENSE, r), p3 = cm::tc2_pick_bn(cm::TC_GROUPED, d);
+        const int p1 = H <= cm::TC2_BIAS_CAP ? cm::tc2_fc1_bn(T, H, d, false, L->num_sms) : 0;
+        const int p2 = cm::tc2_pick_bn(cm::TC_DENSE, r), p3 = cm::tc2_grouped_bn(T, d, 1, (T + 255) / 256, L->num_sms);
         const int b1n = cm::tc_pick_bn(cm::TC_DENSE, H), b2n = cm::tc_pick_bn(cm::TC_DENSE, r);
         const int b3n = cm::tc_pick_bn(cm::TC_GROUPED, d);
         if ((!p1 && !b1n) || (!p2 && !b2n) || (!p3 && !b3n)) return CLEARMOE_EUNSUPPORTED;
@@ -988,6 +990,7 @@ int clearmoe_ffn_forward_scaled(clearmoe_layer* L, const void* x, int64_t T, con
         g.bias = b1;
         g.C = L->z;
         g.ldc = H;
+        g.bn = p1;
         g.epi12 = p1 == 256 && d <= cm::TC2_EPI12_MAX_K;  // short K: the GELU epilogue bounds a tile
         if ((rc = cuda_fail(p1 ? cm::launch_tc_gemm2(g, L->num_sms, s) : cm::launch_tc_gemm(g, L->num_sms, s))))
             return rc;
@@ -1022,6 +1025,7 @@ int clearmoe_ffn_forward_scaled(clearmoe_layer* L, const void* x, int64_t T, con
         if (encode_tmap_bf16(&g3.tmA0, L->t, T, r, 128) || encode_tmap_bf16(&g3.tmB0, U_r, d, r, box3) ||
             encode_tmap_bf16(&g3.tmA1, L->z, T, H, 128) || encode_tmap_bf16(&g3.tmB1[0], R, d, H, box3))
             return CLEARMOE_ECUDA;
+        g3.bn = p3;
         g3.mode = cm::TC_GROUPED;  // one group over all tokens (no offsets): [z | t'] x [R | U_r]
         g3.epi = cm::TC_EPI_STORE;
         g3.M = T;
@@ -1172,8 +1176,8 @@ static int dense_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W
     std::memset(&g, 0, sizeof(g));
     g.status = L->status;
     g.wait_limit_ns = L->wait_limit_ns;
-    const int pair1 = H <= cm::TC2_BIAS_CAP ? cm::tc2_pick_bn(cm::TC_DENSE, H) : 0;  // 2-SM tile widths
-    const int pair2 = cm::tc2_pick_bn(cm::TC_DENSE, d);
+    const int pair1 = H <= cm::TC2_BIAS_CAP ? cm::tc2_fc1_bn(T, H, d, false, L->num_sms) : 0;  // 2-SM tile widths
+    const int pair2 = cm::tc2_grouped_bn(T, d, 1, 0, L->num_sms);
     if (encode_tmap_bf16(&g.tmA0, x, T, d, 128) || encode_tmap_bf16(&g.tmB0, W1, H, d, pair1 ? pair1 / 2 : bn1))
         return CLEARMOE_ECUDA;
     g.mode = cm::TC_DENSE;
@@ -1187,6 +1191,7 @@ static int dense_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W
     g.ln_stats = lns;
     g.ln_colsum = lnc;  // the 1-SM kernel: the column sums in the epilogue
     if (ln && pair1 && (rc = ln_fc1_aug(L, g, T, pair1 / 2))) return rc;  // 2-SM: the augmentation block
+    g.bn = pair1;
     g.epi12 = pair1 == 256 && d <= cm::TC2_EPI12_MAX_K;  // short K: the GELU epilogue bounds a tile
     if ((rc = cuda_fail(pair1 ? cm::launch_tc_gemm2(g, L->num_sms, s) : cm::launch_tc_gemm(g, L->num_sms, s))))
         return rc;
@@ -1197,6 +1202,7 @@ static int dense_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W
     g2.wait_limit_ns = L->wait_limit_ns;
     if (encode_tmap_bf16(&g2.tmA0, L->z, T, H, 128) || encode_tmap_bf16(&g2.tmB0, W2, d, H, pair2 ? pair2 / 2 : bn2))
         return CLEARMOE_ECUDA;
+    g2.bn = pair2;
     g2.mode = cm::TC_DENSE;
     g2.epi = cm::TC_EPI_STORE;
     g2.out_bias = b2;

@@ -215,6 +215,8 @@ struct TcGemmArgs {
     // grouped mode: the z segment's A rows gathered by slot, A row of slot m = a1_rows[m] (perm),
     // by tile::gather4 loads of four rows each; tmA1 then has boxes one row high
     const int32_t* a1_rows;
+    // 2-SM kernel: the pair tile's width (256, 192 or 128, dividing N); 0: tc2_pick_bn(mode, N)
+    int bn;
     // 2-SM dense mode at 256-wide tiles: 12 epilogue warps (three per TMEM lane quarter) and a 160 KB
     // operand ring instead of 8 warps and 192 KB, for short K where the epilogue bounds a tile
     int epi12;
@@ -269,6 +271,11 @@ TcTf32Plan tc_plan_tf32(int N, int K, int64_t m_tiles, int num_sms, int64_t ws_f
 constexpr int TC2_BIAS_CAP = 4096;
 constexpr int TC2_TAB_CAP = 2432;  // routing prefix table entries (ranges x experts)
 int tc2_pick_bn(int mode, int N);
+// The width that fits T: fc1's [T x d] x [H x d] (`slots`: with the routing's slots in its epilogue), and
+// the expert GEMM over G groups (or one: dense fc2) of [T x H] x [d x H], with basis_pairs SM pairs taken by
+// the basis kernel beside it. tc2_pick_bn's or a narrower one; every width gives the same bits.
+int tc2_fc1_bn(int64_t T, int H, int d, bool slots, int num_sms);
+int tc2_grouped_bn(int64_t T, int d, int G, int64_t basis_pairs, int num_sms);
 cudaError_t launch_tc_gemm2(const TcGemmArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_tc_gemm(const TcGemmArgs& a, int num_sms, cudaStream_t s);
 

@@ -744,6 +744,54 @@ int tc2_pick_bn(int mode, int N) {
     return 0;
 }
 
+// fc1's tile width. A round is one tile per SM pair; R256, R192, R128 are the rounds that each width
+// takes. With the routing's slots in its epilogue (`slots`) and K = d > 512 the cost in 256-wide rounds,
+// fitted to whole forwards at 30 sizes, is R256 + 1.33 (the last wide tile's MMAs and epilogue stand
+// alone), 0.844 R192 - 0.39 and 0.6 R128 (a narrow tile brings more operand bytes per column from L2);
+// 192 only with a margin and from five rounds on, where it was the better one throughout. Without the
+// slots a tile's epilogue is shorter and narrow tiles pay up to six rounds. At d <= 512, where 256-wide
+// tiles have twelve epilogue warps: R256 against 0.6 R128.
+// Measured (us, 256 / 192 / 128): ViT-B layer, 3,152 tokens 51.8 / 49.5 / 47.8, 6,304 tokens 76.1 / 74.8 /
+// 72.6, 8,000 tokens 86.2 / 80.9 / 81.9, 12,608 tokens 113.5 / 111.8 / 114.2, 50,432 tokens 378 / 399 / 426;
+// dense ViT-B FFN, 3,152 tokens 37.6 / 32.6 / 33.4, 6,304 tokens 46.2 / 50.6 / 48.8; DeiT-S layer, 197
+// tokens 24.4 / 24.2 / 22.7, 12,608 tokens 51.4 / 57.8 / 55.6.
+int tc2_fc1_bn(int64_t T, int H, int d, bool slots, int num_sms) {
+    const int bn = tc2_pick_bn(TC_DENSE, H);
+    const int64_t pairs = num_sms / 2, mp = (T + 255) / 256;
+    if (bn != 256 || pairs < 1) return bn;
+    auto rounds = [&](int w) { return (mp * (H / w) + pairs - 1) / pairs; };
+    const int64_t r256 = rounds(256), r128 = rounds(128);
+    if (d <= TC2_EPI12_MAX_K) return 3 * r128 < 5 * r256 ? 128 : 256;
+    if (!slots) return r128 <= 6 ? 128 : 256;
+    const double c256 = (double)r256 + 1.33, c128 = 0.6 * (double)r128, best = c128 < c256 ? c128 : c256;
+    if (H % 192 == 0 && r256 >= 5 && 0.844 * (double)rounds(192) - 0.39 + 0.3 < best) return 192;
+    return c128 < c256 ? 128 : 256;
+}
+
+// The tile width of the expert GEMM (and of dense fc2). The blocks are estimated from T (half a block
+// more per group); `basis_pairs` SM pairs run the basis kernel beside it. With R the rounds that blocks x
+// column tiles and the basis take at a width, the cost is u (R + 0.3), u = 1, 0.8, 0.56 for 256, 192, 128
+// columns: a narrow tile's long K chain is shorter, as each K block brings fewer bytes into the SM, but
+// there are more of them. A narrower tile is taken when it is 15 % better by that, and up to three
+// rounds: beyond them all SMs stream from L2 throughout, and the bytes per column decide for the wide tile.
+// Measured (us, 256 / 192 / 128 at d = 768, 192 / 128 at 384): ViT-B layer, 197 tokens 31.2 / 27.6 / 25.1, 3,152
+// tokens 48.2 / 53.9 / 49.9, 4,800 tokens 63.4 / 60.9 / 63.8, 12,608 tokens 113.5 / 119 / 123; folded, 3,152
+// tokens 47.5 / 43.6 / 46.4, 12,608 tokens 111 / 105 / 108; dense FFN, 8,000 tokens 67.0 / 57.5 / 60.1; DeiT-S
+// layer, 788 tokens 24.2 / 22.6, 9,973 tokens 45.0 / 46.7, 12,608 tokens 50.5 / 49.4.
+int tc2_grouped_bn(int64_t T, int d, int G, int64_t basis_pairs, int num_sms) {
+    const int bn = tc2_pick_bn(TC_GROUPED, d);
+    const int64_t pairs = num_sms / 2;
+    if (!bn || pairs < 1) return bn;
+    const int64_t blocks2 = G > 1 ? 2 * T / 256 + G + 1 : 2 * ((T + 255) / 256);  // twice the estimate
+    auto rounds = [&](int w) { return (blocks2 * (d / w) + 2 * basis_pairs + 2 * pairs - 1) / (2 * pairs); };
+    auto cost = [&](int w) { return (w == 256 ? 1.0 : w == 192 ? 0.8 : 0.56) * ((double)rounds(w) + 0.3); };
+    if (rounds(bn) > 3) return bn;
+    int best = bn;
+    for (int w : {192, 128})
+        if (w < bn && d % w == 0 && cost(w) < (best == bn ? 0.85 : 1.0) * cost(best)) best = w;
+    return best;
+}
+
 template <int BN, int MODE, int VAR>
 static cudaError_t launch2(const TcGemmArgs& a, int num_sms, cudaStream_t s) {
     using C = T2v<BN, VAR>;
@@ -780,7 +828,8 @@ static cudaError_t launch2_var(const TcGemmArgs& a, int num_sms, cudaStream_t s)
 }
 
 cudaError_t launch_tc_gemm2(const TcGemmArgs& a, int num_sms, cudaStream_t s) {
-    const int bn = tc2_pick_bn(a.mode, a.N);
+    const int bn = a.bn ? a.bn : tc2_pick_bn(a.mode, a.N);
+    if (a.bn && (a.N % a.bn || (a.bn != 256 && a.bn != 192 && a.bn != 128))) return cudaErrorInvalidValue;
     const bool staged = a.epi == TC_EPI_BIAS_GELU || a.epi == TC_EPI_BIAS_RELU ||
                         a.epi == TC_EPI_SCALE;  // fp32 vector in shared memory
     if (!bn || (staged && (a.mode != TC_DENSE || a.N > TC2_BIAS_CAP))) return cudaErrorInvalidValue;

@@ -140,6 +140,7 @@ struct TcGemmArgs {
     int K1;  // second K segment (grouped only)
     CUtensorMap tmA0, tmA1, tmB0;
     CUtensorMap tmB1[16];
+    CUtensorMap tmB0h, tmB1h[16];  // 2-SM kernel: the B matrices in boxes of half those rows (half tiles)
     const void* gather_src;    // gather: rows of A0 read directly (bf16 [.. x K0])
     int64_t gather_ld;         // elements
     const int32_t* rows;       // gather: A row of output row m; scatter (the 2-SM kernel: whenever
@@ -217,6 +218,8 @@ struct TcGemmArgs {
     const int32_t* a1_rows;
     // 2-SM kernel: the pair tile's width (256, 192 or 128, dividing N); 0: tc2_pick_bn(mode, N)
     int bn;
+    // 2-SM kernel: SM pairs that may run half tiles in the last round
+    int half_pairs;  // <= 0: all
     // 2-SM dense mode at 256-wide tiles: 12 epilogue warps (three per TMEM lane quarter) and a 160 KB
     // operand ring instead of 8 warps and 192 KB, for short K where the epilogue bounds a tile
     int epi12;

@@ -138,6 +138,7 @@ struct PairTile {
     int n0;
     int e;
     bool router;  // the router unit of the pair tile (the router inside fc1)
+    bool half;    // half a pair tile: columns [n0, n0 + BN / 2)
 };
 
 // Kernel variants: the plain dense and grouped GEMMs, the dense GEMM with the router unit (the
@@ -155,13 +156,17 @@ __device__ __forceinline__ int units_per_pair(int n_tiles) {
     return n_tiles + (VAR == TC2_ROUTER ? 1 : 0);
 }
 
+// Units from `full` on are halves: position full + 2 k + h is half h of pair tile full + k.
 template <int BN, int VAR>
-__device__ __forceinline__ PairTile decode_pair(const TcGemmArgs& a, int unit, int n_tiles, const int* s_prefix) {
+__device__ __forceinline__ PairTile decode_pair(const TcGemmArgs& a, int unit, int full, int n_tiles, const int* s_prefix) {
     constexpr int BM = T2<BN>::BM;
     PairTile t;
+    t.half = unit >= full;
+    const int part = t.half ? (unit - full) & 1 : 0;
+    if (t.half) unit = full + ((unit - full) >> 1);
     const int nup = units_per_pair<VAR>(n_tiles);
     const int mp = unit / nup;
-    t.n0 = (unit % nup) * BN;
+    t.n0 = (unit % nup) * BN + part * (BN / 2);
     t.router = VAR == TC2_ROUTER && (unit % nup) == n_tiles;
     if (a.mode == TC_GROUPED) {
         int e = 0;
@@ -357,8 +362,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
         m_pairs = s_prefix[a.E];
     else
         m_pairs = (int)((a.M + 2 * BM - 1) / (2 * BM));
-    const int num_units = warp_uniform(tmem_ok ? m_pairs * units_per_pair<VAR>(n_tiles) : 0);
     const int cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;
+    // Pair tiles, and how many run whole: a last round that would leave more than half of the SM pairs
+    // idle (or a launch with few tiles) runs in half tiles, which take little more than half the time.
+    // half_pairs: beside the basis kernel, only the pairs that start early may take one. Measured
+    // (us): DeiT-S layer with Zipf experts, 9,973 tokens (234 and 86 tiles on 76 pairs) 57.7 -> 53.5; stack of
+    // 12 ViT-B sublayers, 25,216 tokens (309 tiles of each expert GEMM) 2,513 -> 2,488; dense ViT-B FFN, 788
+    // tokens 20.3 -> 19.6. Without the limit a ViT-B layer with class tokens (171 tiles, 50 pairs of
+    // basis) went from 129 to 132.
+    const int num_tiles = warp_uniform(tmem_ok ? m_pairs * units_per_pair<VAR>(n_tiles) : 0);
+    const int tail = (VAR == TC2_PLAIN || VAR == TC2_EPI12) && 2 * (num_tiles % ncl) <= min(ncl, a.half_pairs) ? num_tiles % ncl : 0;
+    const int full = num_tiles - tail, num_units = full + 2 * tail;
 
     if (warp == WARP_TMA) {
         // ------------------------------------------------ producers (both CTAs)
@@ -373,12 +387,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
         uint32_t ph = 0;
         bool ok = true;
         for (int u = cid; u < num_units && ok; u += ncl) {
-            PairTile t = decode_pair<BN, VAR>(a, u, n_tiles, s_prefix);
+            PairTile t = decode_pair<BN, VAR>(a, u, full, n_tiles, s_prefix);
             t.e = warp_uniform(t.e);
             const int am = warp_uniform((int)(t.m0 + (int64_t)rank * BM));
             // the router unit: CTA r supplies W_g rows [16 r, +16) of the 256 x 32 MMA
-            const int bn = t.router ? (int)rank * 16 : t.n0 + (int)rank * BH;
-            const uint32_t stage_tx = t.router ? 2u * (A_BYTES + C::FR_B_BYTES) : 2u * STAGE_BYTES;
+            const int bn = t.router ? (int)rank * 16 : t.n0 + (int)rank * (t.half ? BH / 2 : BH);
+            const uint32_t stage_tx = 2u * (A_BYTES + (t.router ? C::FR_B_BYTES : t.half ? C::B_BYTES / 2 : C::B_BYTES));
             const int nkb_t = (MODE == TC_GROUPED && a.dense_last && t.e == a.E - 1) ? nk1 : nkb;
             int32_t gr[4] = {0, 0, 0, 0};
             if (gather) {  // this lane's four slots; slots past M take the last one (their rows are dropped)
@@ -390,56 +404,47 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                     gr[j] = (uint32_t)tok < (uint64_t)a.M ? tok : 0;  // only a routing that gave up
                 }
             }
-            for (int kb = 0; kb < nkb_t; ++kb) {
-                if (!mbar_wait_warp(empty_bar(stage), ph ^ 1, abort_flag, a.status, lim)) {
-                    ok = false;
-                    break;
+            // K blocks [0, n) of matrices mA and mB, from column 0
+            auto load_blocks = [&](const CUtensorMap* mA, const CUtensorMap* mB, int n, bool gathered) {
+                for (int kb = 0; kb < n; ++kb) {
+                    if (!mbar_wait_warp(empty_bar(stage), ph ^ 1, abort_flag, a.status, lim)) return false;
+                    const uint32_t sA = smem_u32(sm + stage * STAGE_BYTES);
+                    const uint32_t sB = sA + A_BYTES;
+                    const uint32_t fb = full_leader0 + 8u * stage;  // the even CTA's full barrier
+                    if (leader) mbar_arrive_expect_tx_warp(full_bar(stage), stage_tx);
+                    const int kk = kb * BK;
+                    if (gathered)
+                        tma_gather4_pair(sA + 512u * lane, mA, kk, gr[0], gr[1], gr[2], gr[3], fb);
+                    else if (a.a_evict_first)
+                        tma_load_2d_pair_hint(sA, mA, kk, am, fb, pol_a);
+                    else
+                        tma_load_2d_pair(sA, mA, kk, am, fb);
+                    tma_load_2d_pair(sB, mB, kk, bn, fb);
+                    if (++stage == STAGES) {
+                        stage = 0;
+                        ph ^= 1;
+                    }
                 }
-                const uint32_t sA = smem_u32(sm + stage * STAGE_BYTES);
-                const uint32_t sB = sA + A_BYTES;
-                const uint32_t fb = full_leader0 + 8u * stage;  // the even CTA's full barrier
-                if (leader) mbar_arrive_expect_tx_warp(full_bar(stage), stage_tx);
-                const CUtensorMap* mA;
-                const CUtensorMap* mB;
-                int kk;
-                bool gathered = false;
-                if (MODE != TC_GROUPED) {  // x x W (or x x W_g), then the augmentation block
-                    mA = kb < nk0 ? &a.tmA0 : &a.tmA1;
-                    mB = t.router ? &a.tmR : kb < nk0 ? &a.tmB0 : &a.tmB1[0];
-                    kk = kb < nk0 ? kb * BK : 0;
-                } else if (kb < nk1) {  // z x W_e^res
-                    mA = &a.tmA1;
-                    mB = &a.tmB1[t.e];
-                    kk = kb * BK;
-                    gathered = gather;
-                } else {  // t x U_r
+                return true;
+            };
+            if (MODE != TC_GROUPED) {  // x x W (or x x W_g), then the augmentation block
+                ok = load_blocks(&a.tmA0, t.router ? &a.tmR : t.half ? &a.tmB0h : &a.tmB0, nk0, false);
+                if (ok && nk1 > 0) ok = load_blocks(&a.tmA1, t.half ? &a.tmB1h[0] : &a.tmB1[0], nk1, false);
+            } else {  // z x W_e^res, then t x U_r
+                ok = load_blocks(&a.tmA1, t.half ? &a.tmB1h[t.e] : &a.tmB1[t.e], nk1, gather);
+                if (ok && nkb_t > nk1) {
                     if (!waited) {
                         pdl_wait();
                         waited = true;
                     }
-                    mA = &a.tmA0;
-                    mB = &a.tmB0;
-                    kk = (kb - nk1) * BK;
-                }
-                if (gathered) {
-                    tma_gather4_pair(sA + 512u * lane, mA, kk, gr[0], gr[1], gr[2], gr[3], fb);
-                } else {
-                    if (a.a_evict_first)
-                        tma_load_2d_pair_hint(sA, mA, kk, am, fb, pol_a);
-                    else
-                        tma_load_2d_pair(sA, mA, kk, am, fb);
-                }
-                tma_load_2d_pair(sB, mB, kk, bn, fb);
-                if (++stage == STAGES) {
-                    stage = 0;
-                    ph ^= 1;
+                    ok = load_blocks(&a.tmA0, t.half ? &a.tmB0h : &a.tmB0, nk0, false);
                 }
             }
         }
     } else if (warp == WARP_MMA) {
         // ------------------------------------------------ MMA issuer (even CTA, the whole warp)
         if (leader) {
-            const uint32_t idesc_t = idesc_bf16_f32(2 * BM, BN);
+            const uint32_t idesc_t = idesc_bf16_f32(2 * BM, BN), idesc_h = idesc_bf16_f32(2 * BM, BN / 2);
             const uint32_t idesc_r = idesc_bf16_f32(2 * BM, 32);  // the router unit: 256 x 32
             const int nup = units_per_pair<VAR>(n_tiles);
             // Stage s's descriptors are the stage-0 ones plus the byte offset / 16 in the start
@@ -454,9 +459,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                 if (!mbar_wait_warp(tempty_bar(acc), aph ^ 1, abort_flag, a.status, lim)) break;
                 tc_fence_after();
                 const uint32_t dtm = tmem_base + acc * BN;
-                const uint32_t idesc = (VAR == TC2_ROUTER && u % nup == n_tiles) ? idesc_r : idesc_t;
+                const uint32_t idesc = (VAR == TC2_ROUTER && u % nup == n_tiles) ? idesc_r : u >= full ? idesc_h : idesc_t;
                 int nkb_t = nkb;  // the dense path's group: the z x W2 segment alone
-                if (MODE == TC_GROUPED && a.dense_last && warp_uniform(decode_pair<BN, VAR>(a, u, n_tiles, s_prefix).e) == a.E - 1)
+                if (MODE == TC_GROUPED && a.dense_last && warp_uniform(decode_pair<BN, VAR>(a, u, full, n_tiles, s_prefix).e) == a.E - 1)
                     nkb_t = nk1;
                 for (int kb = 0; kb < nkb_t; ++kb) {
                     if (!mbar_wait_warp(full_bar(stage), ph, abort_flag, a.status, lim)) {
@@ -499,9 +504,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
     } else if (warp < NUM_EPI) {
         // ------------------------------------------------ epilogue (both CTAs, own 128 rows)
         const int q = warp & 3;  // a warp reads the TMEM lanes of its index mod 4
-        // this warp's columns of every tile: chunks [grp NCH / GROUPS, (grp + 1) NCH / GROUPS)
         const int grp = warp >> 2;
-        const int c_lo = CW * (grp * C::NCH / C::GROUPS), c_hi = CW * ((grp + 1) * C::NCH / C::GROUPS);
         unsigned char* wstg = stg + warp * 32 * STG_ROW;
         // Staging by half warps: the 16 rows of lanes 16 h .. 16 h + 15 as 64-byte rows (a 32-column
         // chunk), 16-byte piece j of row r at piece j ^ ((r >> 1) & 3) (conflict-free for the
@@ -513,7 +516,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
         uint32_t aph = 0;
         int fr_it = 0;  // router units handled so far (the router inside fc1)
         for (int u = cid; u < num_units; u += ncl) {
-            const PairTile t = decode_pair<BN, VAR>(a, u, n_tiles, s_prefix);
+            const PairTile t = decode_pair<BN, VAR>(a, u, full, n_tiles, s_prefix);
+            // this warp's columns of the tile: chunks [grp n / GROUPS, (grp + 1) n / GROUPS) of its n
+            const int nch = t.half ? C::NCH / 2 : C::NCH;
+            const int c_lo = CW * (grp * nch / C::GROUPS), c_hi = CW * ((grp + 1) * nch / C::GROUPS);
             const int64_t mrow = t.m0 + (int64_t)rank * BM + q * 32 + lane;
             // the token's routing word, loaded before the accumulator wait so that the wait hides it
             const uint32_t rtw = (MODE == TC_DENSE && a.rt_info && mrow < t.hi) ? (uint32_t)a.rt_info[mrow] : 0u;
@@ -527,7 +533,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                 // (lowest index on ties), count each expert's rows of the quarter by ballots, and
                 // exchange the counts through shared memory (a barrier per buffer, bounded waits):
                 // rank = earlier quarters' rows of the expert + earlier lanes' of this quarter.
-                if (c_lo == 0) {
+                if (grp == 0) {
                     const int E = a.fr_E;
                     const int rb = fr_it & 1;
                     int* rc = s_frc + rb * 4 * CM_MAX_E;
@@ -586,7 +592,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                         else if (e < a.rt_E)
                             orow = (int64_t)s_off[e] + s_tab[rc * a.rt_E + e] + (int)(w >> 8);
                         if ((uint64_t)orow >= (uint64_t)a.M) orow = -1;  // only a routing that gave up
-                        if (orow >= 0 && t.n0 == 0 && c_lo == 0) a.rt_perm[orow] = (int32_t)mrow;  // once per token
+                        if (orow >= 0 && t.n0 == 0 && grp == 0) a.rt_perm[orow] = (int32_t)mrow;  // once per token
                     } else {
                         orow = a.rows ? (int64_t)a.rows[mrow] : mrow;
                         if ((uint64_t)orow >= (uint64_t)a.M) orow = -1;  // only a routing that gave up
@@ -793,7 +799,8 @@ int tc2_grouped_bn(int64_t T, int d, int G, int64_t basis_pairs, int num_sms) {
 }
 
 template <int BN, int MODE, int VAR>
-static cudaError_t launch2(const TcGemmArgs& a, int num_sms, cudaStream_t s) {
+static cudaError_t launch2(TcGemmArgs a, int num_sms, cudaStream_t s) {
+    if (a.half_pairs <= 0) a.half_pairs = num_sms / 2;
     using C = T2v<BN, VAR>;
     const void* fn = (const void*)tc_gemm2_kernel<BN, MODE, VAR>;
     const cudaError_t e = smem_attr_once(fn, C::SMEM);

@@ -321,7 +321,7 @@ int clearmoe_set_profile_events(clearmoe_layer* layer, void* const* events, int3
  *   - The first call on a device looks up the array's device address (once per device, with that
  *     device current); make that first call before any stream capture.
  *   - Every call shares the array and it keeps the last call's contents; each call clears what
- *     must start at zero (the status words; the histograms are rewritten before they are read).
+ *     must start at zero (the caller's status word; the histograms are rewritten before they are read).
  *     Calls whose work overlaps on the GPU (other streams, other host threads) race on the
  *     array: serialise them.
  *   - status (optional int32 device pointer, else NULL) is set to 0 at the start of the call and

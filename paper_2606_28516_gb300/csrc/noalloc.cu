@@ -87,10 +87,11 @@ extern "C" int clearmoe_route_noalloc(const void* x, int64_t T, int32_t d, int32
     if (grid > kNoallocMaxCtas) return CLEARMOE_EUNSUPPORTED;  // beyond the scratch's capacity
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // Only the spare status word and the caller's status start at zero; the histograms are
-    // fully rewritten by every launch before they are read.
-    if (cudaMemsetAsync(scratch + 2, 0, sizeof(int32_t), s) != cudaSuccess ||
-        (status && cudaMemsetAsync(status, 0, sizeof(int32_t), s) != cudaSuccess)) {
+    // Only the caller's status starts at zero: the spare word is never read, and the histograms are
+    // fully rewritten by every launch before they are read. Clearing the spare word too was a memset
+    // node ahead of the two kernels, which also kept the first from starting early: 50,432 tokens of
+    // d = 768, back to back, 24.0 us a call with it, 18.5 without.
+    if (status && cudaMemsetAsync(status, 0, sizeof(int32_t), s) != cudaSuccess) {
         (void)cudaGetLastError();
         return CLEARMOE_ECUDA;
     }

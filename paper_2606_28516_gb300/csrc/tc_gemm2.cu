@@ -42,8 +42,9 @@ struct T2 {
     // chunks of the tile of epilogue warp group g (the warps g * 4 .. g * 4 + 3): [g NCH / G, (g + 1) NCH / G)
     static constexpr int GROUPS = NUM_EPI / 4;
     // Staging: 1 KB per epilogue warp (32 x STG_ROW bytes), which each half warp in turn fills
-    // with its 16 rows of one 32-column chunk as 64-byte rows (layout at the epilogue).
-    static constexpr int STG_ROW = 32;
+    // with its 16 rows of one 32-column chunk as 64-byte rows (layout at the epilogue); 2 KB with twelve
+    // warps, for all 32 rows.
+    static constexpr int STG_ROW = NEPI_ == 8 ? 32 : 64;
     static constexpr int STG_BYTES = NUM_EPI * 32 * STG_ROW;
     static constexpr int BIAS_CAP = TC2_BIAS_CAP;         // fp32 bias / scale staged in shared memory
     static constexpr int TAB_CAP = TC2_TAB_CAP;           // routing prefix table (fused fc1)
@@ -144,9 +145,15 @@ struct PairTile {
 // Kernel variants: the plain dense and grouped GEMMs, the dense GEMM with the router unit (the
 // router inside fc1), and the grouped GEMM whose z rows are gathered by slot. Each variant is its own
 // instantiation, so the plain kernels carry none of the others' code.
-enum Tc2Var { TC2_PLAIN = 0, TC2_ROUTER = 1, TC2_GATHER = 2, TC2_EPI12 = 3 };
-// TC2_EPI12: the plain dense GEMM with 12 epilogue warps (three per TMEM lane quarter) and a 160 KB
-// operand ring, for short K (fc1 at d <= 512), where the epilogue's GELU bounds a tile.
+enum Tc2Var { TC2_PLAIN = 0, TC2_ROUTER = 1, TC2_GATHER = 2, TC2_EPI12 = 3, TC2_FC1 = 4 };
+// TC2_FC1: the dense GEMM whose epilogue is bias + GELU to bf16 rows (rstd of a folded LayerNorm
+// included) and nothing else. The options of the general epilogue (its kind, row and column scales,
+// fp32 rows, column sums), tested per 32-column chunk, cost the epilogue warps a tenth of fc1 at every
+// size, and their schedulers' issue slots and energy with it: DeiT-B layer at 50,432 tokens, fc1 181 ->
+// 160 us and the layer 381 -> 349; dense FFN at 100,864 tokens 583 -> 544 us. TC2_EPI12: the same with
+// 12 epilogue warps (three per TMEM lane quarter), each staging its 32 rows at once, and a 160 KB operand
+// ring, for short K (fc1 at d <= 512), where the epilogue bounds a tile: DeiT-S layer at 12,608 tokens
+// 52.5 us with the options, 50.3 without, 48.3 with whole-warp staging.
 template <int BN, int VAR>
 using T2v = T2<BN, VAR == TC2_EPI12 ? 12 : 8>;
 
@@ -371,7 +378,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
     // tokens 20.3 -> 19.6. Without the limit a ViT-B layer with class tokens (171 tiles, 50 pairs of
     // basis) went from 129 to 132.
     const int num_tiles = warp_uniform(tmem_ok ? m_pairs * units_per_pair<VAR>(n_tiles) : 0);
-    const int tail = (VAR == TC2_PLAIN || VAR == TC2_EPI12) && 2 * (num_tiles % ncl) <= min(ncl, a.half_pairs) ? num_tiles % ncl : 0;
+    const int tail = VAR != TC2_ROUTER && VAR != TC2_GATHER && 2 * (num_tiles % ncl) <= min(ncl, a.half_pairs) ? num_tiles % ncl : 0;
     const int full = num_tiles - tail, num_units = full + 2 * tail;
 
     if (warp == WARP_TMA) {
@@ -510,7 +517,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
         // chunk), 16-byte piece j of row r at piece j ^ ((r >> 1) & 3) (conflict-free for the
         // row-wise writes and the 4-lanes-per-row reads); each store instruction then writes
         // 8 rows x 64 contiguous bytes.
-        static_assert(CW == 32 && 16 * 64 == 32 * STG_ROW, "a half warp's 64-byte rows fill the warp's staging");
+        // With STG_ROW = 64 both halves' rows are staged at once.
+        static_assert(CW == 32 && 16 * 64 <= 32 * STG_ROW, "a half warp's 64-byte rows fit the warp's staging");
+        // options that this instantiation's epilogue never has
+        constexpr bool FC1 = VAR == TC2_FC1 || VAR == TC2_EPI12;
         const uint32_t tempty_leader0 = map_to_rank(tempty_bar(0), 0);
         int acc = 0;
         uint32_t aph = 0;
@@ -598,7 +608,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                         if ((uint64_t)orow >= (uint64_t)a.M) orow = -1;  // only a routing that gave up
                     }
                 }
-                const float rsc = (a.group_scale && mrow < t.hi) ? tc_row_scale(a, mrow) : 1.f;
+                const float rsc = (!FC1 && a.group_scale && mrow < t.hi) ? tc_row_scale(a, mrow) : 1.f;
                 // with the mean term in the accumulator (augmentation block) the bias add also scales by
                 // rstd: fma(acc, 1, b) = acc + b exactly, so without the LayerNorm nothing changes
                 const float lns = (a.ln_stats && !a.ln_colsum) ? ln.y : 1.f;
@@ -608,8 +618,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                 uint16_t* dst_row[4];
     #pragma unroll
                 for (int hp = 0; hp < 4; ++hp) {
-                    const int64_t o = __shfl_sync(0xffffffffu, orow, 8 * hp + lane / 4);
-                    dst_row[hp] = o >= 0 ? static_cast<uint16_t*>(a.C) + o * a.ldc + t.n0 + (lane % 4) * 8 : nullptr;
+                    const int o = __shfl_sync(0xffffffffu, (int)orow, 8 * hp + lane / 4);  // rows < 2^30
+                    dst_row[hp] = o >= 0 ? static_cast<uint16_t*>(a.C) + (int64_t)o * a.ldc + t.n0 + (lane % 4) * 8 : nullptr;
                 }
                 for (int c = c_lo; c < c_hi; c += CW) {
                     uint32_t v[CW];
@@ -621,7 +631,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
     #pragma unroll
                     for (int j = 0; j < CW; ++j) f[j] = __uint_as_float(v[j]);
                     const int nb = t.n0 + c;
-                    if (a.ln_stats && a.ln_colsum) {  // W LN(y) = rstd (W y - mean c), c_n = sum_k W[n, k]
+                    if (MODE == TC_DENSE && !FC1 && a.ln_stats && a.ln_colsum) {  // W LN(y) = rstd (W y - mean c), c_n = sum_k W[n, k]
                         const float4* cp = reinterpret_cast<const float4*>(a.ln_colsum + nb);  // same for all lanes
     #pragma unroll
                         for (int j4 = 0; j4 < CW / 4; ++j4) {
@@ -632,7 +642,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                             f[4 * j4 + 3] = ln.y * fmaf(-ln.x, c4.w, f[4 * j4 + 3]);
                         }
                     }
-                    if (a.epi == TC_EPI_BIAS_GELU) {
+                    if (FC1 || (MODE == TC_DENSE && a.epi == TC_EPI_BIAS_GELU)) {
                         const float4* bp = reinterpret_cast<const float4*>(s_bias + nb);  // same for all lanes
     #pragma unroll
                         for (int j4 = 0; j4 < CW / 4; ++j4) {
@@ -646,7 +656,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                             f[4 * j4 + 2] = g1.x;
                             f[4 * j4 + 3] = g1.y;
                         }
-                    } else if (a.epi == TC_EPI_BIAS_RELU) {
+                    } else if (MODE == TC_DENSE && a.epi == TC_EPI_BIAS_RELU) {
                         const float4* bp = reinterpret_cast<const float4*>(s_bias + nb);  // same for all lanes
     #pragma unroll
                         for (int j4 = 0; j4 < CW / 4; ++j4) {
@@ -668,7 +678,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                             f[4 * j4 + 2] = p1.x;
                             f[4 * j4 + 3] = p1.y;
                         }
-                    } else if (a.epi == TC_EPI_SCALE) {
+                    } else if (MODE == TC_DENSE && a.epi == TC_EPI_SCALE) {
                         const float4* sp = reinterpret_cast<const float4*>(s_bias + nb);  // same for all lanes
     #pragma unroll
                         for (int j4 = 0; j4 < CW / 4; ++j4) {
@@ -681,7 +691,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                             f[4 * j4 + 3] = p1.y;
                         }
                     }
-                    if (a.group_scale) {
+                    if (!FC1 && a.group_scale) {
     #pragma unroll
                         for (int j2 = 0; j2 < CW / 2; ++j2) {
                             const float2 p2 = __fmul2_rn(make_float2(f[2 * j2], f[2 * j2 + 1]), make_float2(rsc, rsc));
@@ -689,7 +699,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                             f[2 * j2 + 1] = p2.y;
                         }
                     }
-                    if (a.c_f32) {  // fp32 output: each lane stores its row's 32 values as computed
+                    if (MODE == TC_DENSE && !FC1 && a.c_f32) {  // fp32 output: each lane stores its row's 32 values as computed
                         if (orow >= 0) {
                             float4* dstf = reinterpret_cast<float4*>(static_cast<float*>(a.C) + orow * a.ldc + nb);
     #pragma unroll
@@ -698,28 +708,36 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                         }
                         continue;
                     }
+                    auto stage_row = [&](int rw) {  // this lane's row as staged row rw
+                        unsigned char* dst = wstg + rw * 64;
     #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        if ((lane >> 4) == h) {
-                            const int rw = lane & 15;
-                            unsigned char* dst = wstg + rw * 64;
-    #pragma unroll
-                            for (int j8 = 0; j8 < 4; ++j8) {
-                                const float* g = f + 8 * j8;
-                                *reinterpret_cast<uint4*>(dst + ((j8 ^ ((rw >> 1) & 3)) << 4)) =
-                                    make_uint4(pack_bf16(g[0], g[1]), pack_bf16(g[2], g[3]), pack_bf16(g[4], g[5]),
-                                               pack_bf16(g[6], g[7]));
-                            }
+                        for (int j8 = 0; j8 < 4; ++j8) {
+                            const float* g = f + 8 * j8;
+                            *reinterpret_cast<uint4*>(dst + ((j8 ^ ((rw >> 1) & 3)) << 4)) =
+                                make_uint4(pack_bf16(g[0], g[1]), pack_bf16(g[2], g[3]), pack_bf16(g[4], g[5]),
+                                           pack_bf16(g[6], g[7]));
                         }
+                    };
+                    auto store_rows = [&](int rr, uint16_t* dst) {  // 8 staged rows, this lane's piece of row rr
+                        const int ch = (lane % 4) ^ ((rr >> 1) & 3);
+                        const uint4 val = *reinterpret_cast<const uint4*>(wstg + rr * 64 + ch * 16);
+                        if (dst) *reinterpret_cast<uint4*>(dst + c) = val;
+                    };
+                    if constexpr (STG_ROW == 64) {
+                        stage_row(lane);
                         __syncwarp();
     #pragma unroll
-                        for (int p = 0; p < 2; ++p) {
-                            const int rr = 8 * p + lane / 4;  // row of the half
-                            const int ch = (lane % 4) ^ ((rr >> 1) & 3);
-                            const uint4 val = *reinterpret_cast<const uint4*>(wstg + rr * 64 + ch * 16);
-                            if (dst_row[2 * h + p]) *reinterpret_cast<uint4*>(dst_row[2 * h + p] + c) = val;
-                        }
+                        for (int hp = 0; hp < 4; ++hp) store_rows(8 * hp + lane / 4, dst_row[hp]);
                         __syncwarp();
+                    } else {
+    #pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            if ((lane >> 4) == h) stage_row(lane & 15);
+                            __syncwarp();
+    #pragma unroll
+                            for (int p = 0; p < 2; ++p) store_rows(8 * p + lane / 4, dst_row[2 * h + p]);
+                            __syncwarp();
+                        }
                     }
                 }
             }
@@ -750,52 +768,50 @@ int tc2_pick_bn(int mode, int N) {
     return 0;
 }
 
-// fc1's tile width. A round is one tile per SM pair; R256, R192, R128 are the rounds that each width
-// takes. With the routing's slots in its epilogue (`slots`) and K = d > 512 the cost in 256-wide rounds,
-// fitted to whole forwards at 30 sizes, is R256 + 1.33 (the last wide tile's MMAs and epilogue stand
-// alone), 0.844 R192 - 0.39 and 0.6 R128 (a narrow tile brings more operand bytes per column from L2);
-// 192 only with a margin and from five rounds on, where it was the better one throughout. Without the
-// slots a tile's epilogue is shorter and narrow tiles pay up to six rounds. At d <= 512, where 256-wide
-// tiles have twelve epilogue warps: R256 against 0.6 R128.
-// Measured (us, 256 / 192 / 128): ViT-B layer, 3,152 tokens 51.8 / 49.5 / 47.8, 6,304 tokens 76.1 / 74.8 /
-// 72.6, 8,000 tokens 86.2 / 80.9 / 81.9, 12,608 tokens 113.5 / 111.8 / 114.2, 50,432 tokens 378 / 399 / 426;
-// dense ViT-B FFN, 3,152 tokens 37.6 / 32.6 / 33.4, 6,304 tokens 46.2 / 50.6 / 48.8; DeiT-S layer, 197
-// tokens 24.4 / 24.2 / 22.7, 12,608 tokens 51.4 / 57.8 / 55.6.
+// fc1's tile width: 256, or 128 while those take few rounds (a round is one tile per SM pair). With the
+// routing's slots in the epilogue 128-wide tiles win only when one round holds them all (their
+// epilogues, which end the kernel, are half as long); without the slots up to six rounds, or two at
+// d <= 512, where the 256-wide kernel has twelve epilogue warps. From there on a wide tile's operand
+// bytes per column decide, and half tiles fill its last round.
+// Measured (us, 256 / 128): DeiT-S layer, 197 tokens 21.8 / 21.0, 1,200 tokens 23.5 / 22.5, 2,400 tokens 25.1 /
+// 25.8, 9,973 tokens 41.3 / 44.3; d = 1,024 layer, 500 tokens 34.4 / 32.7, 4,000 tokens 65.0 / 67.7; ViT-B layer,
+// 3,152 tokens 46.6 / 47.5, 25,216 tokens 186 / 222; dense ViT-B FFN, 788 tokens 20.8 / 19.3, 4,000 tokens 35.4 /
+// 34.2, 12,608 tokens 83.2 / 90.5; dense DeiT-S FFN, 1,200 tokens 16.3 / 13.4, 5,000 tokens 20.6 / 20.9.
 int tc2_fc1_bn(int64_t T, int H, int d, bool slots, int num_sms) {
     const int bn = tc2_pick_bn(TC_DENSE, H);
-    const int64_t pairs = num_sms / 2, mp = (T + 255) / 256;
+    const int64_t pairs = num_sms / 2;
     if (bn != 256 || pairs < 1) return bn;
-    auto rounds = [&](int w) { return (mp * (H / w) + pairs - 1) / pairs; };
-    const int64_t r256 = rounds(256), r128 = rounds(128);
-    if (d <= TC2_EPI12_MAX_K) return 3 * r128 < 5 * r256 ? 128 : 256;
-    if (!slots) return r128 <= 6 ? 128 : 256;
-    const double c256 = (double)r256 + 1.33, c128 = 0.6 * (double)r128, best = c128 < c256 ? c128 : c256;
-    if (H % 192 == 0 && r256 >= 5 && 0.844 * (double)rounds(192) - 0.39 + 0.3 < best) return 192;
-    return c128 < c256 ? 128 : 256;
+    const int64_t r128 = ((T + 255) / 256 * (H / 128) + pairs - 1) / pairs;
+    return r128 <= (slots ? 1 : d <= TC2_EPI12_MAX_K ? 2 : 6) ? 128 : 256;
 }
 
-// The tile width of the expert GEMM (and of dense fc2). The blocks are estimated from T (half a block
-// more per group); `basis_pairs` SM pairs run the basis kernel beside it. With R the rounds that blocks x
-// column tiles and the basis take at a width, the cost is u (R + 0.3), u = 1, 0.8, 0.56 for 256, 192, 128
-// columns: a narrow tile's long K chain is shorter, as each K block brings fewer bytes into the SM, but
-// there are more of them. A narrower tile is taken when it is 15 % better by that, and up to three
-// rounds: beyond them all SMs stream from L2 throughout, and the bytes per column decide for the wide tile.
-// Measured (us, 256 / 192 / 128 at d = 768, 192 / 128 at 384): ViT-B layer, 197 tokens 31.2 / 27.6 / 25.1, 3,152
-// tokens 48.2 / 53.9 / 49.9, 4,800 tokens 63.4 / 60.9 / 63.8, 12,608 tokens 113.5 / 119 / 123; folded, 3,152
-// tokens 47.5 / 43.6 / 46.4, 12,608 tokens 111 / 105 / 108; dense FFN, 8,000 tokens 67.0 / 57.5 / 60.1; DeiT-S
-// layer, 788 tokens 24.2 / 22.6, 9,973 tokens 45.0 / 46.7, 12,608 tokens 50.5 / 49.4.
+// The tile width of the expert GEMM (and of dense fc2), from the pair tiles that T rows in G groups give
+// (the routing is not known here: even groups, or half a block more per group) and the SM pairs that
+// the basis kernel takes beside it. While one round holds a width's tiles, the narrowest such width: a
+// tile's long K chain bounds the kernel, and a narrow one's is shorter. Otherwise the widest (operand
+// bytes per column), except that beside the basis a few tiles over a whole number of rounds, which no
+// early pair can take as halves, are better cut into the next narrower width, up to two rounds.
+// Measured (us, 256 / 192 / 128 at d = 768, 256 / 128 at 512 and 1,024, 192 / 128 at 384): dense FFN, 788 tokens
+// 26.1 / 22.6 / 19.3, 6,304 tokens 44.4 / 45.6 / 44.6; folded layer, 3,152 tokens 42.3 / 39.7 / 42.8, 25,216 tokens
+// 163 / 171 / 190; ViT-B layer, 1,576 tokens 36.9 / 33.7 / 32.6, 3,152 tokens 45.9 / 52.0 / 48.3, 4,800 tokens (91
+// pair tiles with the basis on 76 pairs) 59.3 / 56.2 / 59.8, 8,000 tokens (128) 72.2 / 81.3 / 74.7; d = 1,024,
+// 4,000 tokens (80) 73.4 / 64.3; d = 512, 7,000 tokens (84) 44.3 / 40.8; DeiT-S layer, 9,973 tokens (119) 41.0 /
+// 42.4, 12,608 tokens (154) 46.9 / 45.4.
 int tc2_grouped_bn(int64_t T, int d, int G, int64_t basis_pairs, int num_sms) {
     const int bn = tc2_pick_bn(TC_GROUPED, d);
     const int64_t pairs = num_sms / 2;
     if (!bn || pairs < 1) return bn;
-    const int64_t blocks2 = G > 1 ? 2 * T / 256 + G + 1 : 2 * ((T + 255) / 256);  // twice the estimate
-    auto rounds = [&](int w) { return (blocks2 * (d / w) + 2 * basis_pairs + 2 * pairs - 1) / (2 * pairs); };
-    auto cost = [&](int w) { return (w == 256 ? 1.0 : w == 192 ? 0.8 : 0.56) * ((double)rounds(w) + 0.3); };
-    if (rounds(bn) > 3) return bn;
-    int best = bn;
-    for (int w : {192, 128})
-        if (w < bn && d % w == 0 && cost(w) < (best == bn ? 0.85 : 1.0) * cost(best)) best = w;
-    return best;
+    const int64_t even = (T + (int64_t)256 * G - 1) / ((int64_t)256 * G) * G;  // G equal groups
+    const int64_t some = (2 * T + (int64_t)256 * G + 511) / 512;                // half a block more per group
+    const int64_t blocks = G > 1 && some > even ? some : even;
+    int next = bn;  // the next narrower width
+    for (int w : {128, 192})
+        if (w < bn && d % w == 0) {
+            if (blocks * (d / w) + basis_pairs <= pairs) return w;
+            next = w;
+        }
+    const int64_t tiles = blocks * (d / bn) + basis_pairs, rounds = tiles / pairs, over = tiles % pairs;
+    return basis_pairs > 0 && rounds >= 1 && rounds <= 2 && over > 0 && 5 * over <= pairs ? next : bn;
 }
 
 template <int BN, int MODE, int VAR>
@@ -828,9 +844,12 @@ template <int BN>
 static cudaError_t launch2_var(const TcGemmArgs& a, int num_sms, cudaStream_t s) {
     if (a.mode == TC_GROUPED)
         return a.a1_rows ? launch2<BN, TC_GROUPED, TC2_GATHER>(a, num_sms, s) : launch2<BN, TC_GROUPED, TC2_PLAIN>(a, num_sms, s);
+    // bias + GELU to bf16 and nothing else: fc1's own instantiations
+    const bool fc1 = a.epi == TC_EPI_BIAS_GELU && !a.c_f32 && !a.group_scale && !(a.ln_stats && a.ln_colsum) && a.fr_E == 0;
     if constexpr (BN == 256) {
-        if (a.epi12) return launch2<BN, TC_DENSE, TC2_EPI12>(a, num_sms, s);
+        if (a.epi12) return fc1 ? launch2<BN, TC_DENSE, TC2_EPI12>(a, num_sms, s) : cudaErrorInvalidValue;
     }
+    if (fc1) return launch2<BN, TC_DENSE, TC2_FC1>(a, num_sms, s);
     return a.fr_E > 0 ? launch2<BN, TC_DENSE, TC2_ROUTER>(a, num_sms, s) : launch2<BN, TC_DENSE, TC2_PLAIN>(a, num_sms, s);
 }
 

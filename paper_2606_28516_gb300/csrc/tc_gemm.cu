@@ -657,7 +657,7 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
                         const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
                         for (int h = 0; h < 4; ++h) {
-                            const float2 g = gelu_pair_as(
+                            const float2 g = gelu_pair_bf16(
                                 __fadd2_rn(make_float2(f[j8 * 8 + 2 * h], f[j8 * 8 + 2 * h + 1]),
                                            make_float2(bf16_lo(bw[h]), bf16_hi(bw[h]))));
                             f[j8 * 8 + 2 * h] = g.x;

@@ -647,9 +647,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
     #pragma unroll
                         for (int j4 = 0; j4 < CW / 4; ++j4) {
                             const float4 b = bp[j4];
-                            const float2 g0 = gelu_pair_as(
+                            const float2 g0 = gelu_pair_bf16(
                                 __ffma2_rn(make_float2(f[4 * j4], f[4 * j4 + 1]), lns2, make_float2(b.x, b.y)));
-                            const float2 g1 = gelu_pair_as(
+                            const float2 g1 = gelu_pair_bf16(
                                 __ffma2_rn(make_float2(f[4 * j4 + 2], f[4 * j4 + 3]), lns2, make_float2(b.z, b.w)));
                             f[4 * j4] = g0.x;
                             f[4 * j4 + 1] = g0.y;

@@ -553,7 +553,15 @@ int route_max_ctas(int num_sms, int, int, int) { return min(num_sms * 8, 32 * RT
 int route_grid(int64_t T, int d, int E, int dtype, int num_sms, int* grid, int* chunk) {
     const bool bf16 = dtype == CLEARMOE_BF16;
     int occ = 0;
-    int64_t want = (int64_t)num_sms * (bf16 ? 1 : 2);  // bf16: one CTA per SM owns the ring
+    // bf16: one CTA per SM owns the ring. fp32: two per SM, but no more ranges than fc1's prefix table takes
+    // (256, and TC2_TAB_CAP entries of ranges x experts). The slots are then formed in fc1's epilogue, and the
+    // slot kernel, which the 304 ranges of two CTAs on every SM needed, is not launched: 5.3 us by itself;
+    // the DeiT-T layer at 12,608 tokens goes from 86 to 83.9 us.
+    int64_t want = num_sms;
+    if (!bf16) {
+        const int64_t fit = TC2_TAB_CAP / (E > 0 ? E : 1) < 256 ? TC2_TAB_CAP / (E > 0 ? E : 1) : 256;
+        want = fit > num_sms ? (fit < 2 * num_sms ? fit : 2 * num_sms) : num_sms;
+    }
     // equal ranges over all CTAs (a range's last block may be partial)
     int64_t ch = (T + want - 1) / want;
     // the shared-memory attribute belongs to a device: set once per device

@@ -224,12 +224,19 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
     const int nk0 = (a.K0 + KE - 1) / KE;
     const int nk1 = MODE == TC_GROUPED ? (a.K1 + KE - 1) / KE : 0;
     const int nkb = nk0 + nk1;
-    // K blocks [lo, hi) of a unit: the tile's blocks [kb0, nkb) (kb0 = nk0 for the class tokens' group)
+    // fp32 grouped: the z segment (K1) first, then t's (K0), which the preceding basis kernel may still
+    // be writing; bf16: t's first
+    constexpr bool Z_FIRST = TF32 && MODE == TC_GROUPED;
+    auto in_k0 = [&](int kb) { return Z_FIRST ? kb >= nk1 : kb < nk0; };
+    // block kb's index within its segment
+    auto seg_block = [&](int kb) { return Z_FIRST ? (kb >= nk1 ? kb - nk1 : kb) : (kb < nk0 ? kb : kb - nk0); };
+    // K blocks [lo, hi) of a unit: the tile's blocks (the z segment's alone for the class tokens' group)
     // cut into ksp equal ranges, range sp of them
     auto k_range = [&](const TileInfo& t, int sp, int& lo, int& hi) {
-        const int kb0 = (MODE == TC_GROUPED && a.dense_last && t.e == a.E - 1) ? nk0 : 0;
-        lo = kb0 + (nkb - kb0) * sp / ksp;
-        hi = kb0 + (nkb - kb0) * (sp + 1) / ksp;
+        const bool z_only = MODE == TC_GROUPED && a.dense_last && t.e == a.E - 1;
+        const int kb0 = z_only && !Z_FIRST ? nk0 : 0, n = z_only ? nk1 : nkb;
+        lo = kb0 + n * sp / ksp;
+        hi = kb0 + n * (sp + 1) / ksp;
     };
 
     if (threadIdx.x == 0) {
@@ -254,8 +261,9 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // everything above overlaps the predecessor kernel; from here on its results are read
-    pdl_wait();
+    // everything above overlaps the predecessor kernel; from here on its results are read (fp32: by every
+    // thread, or by the roles that read them, see pdl_wait_role)
+    if (!TF32 || a.pdl_wait_role == 0 || (a.pdl_wait_role == 1 && warp < TC_NUM_EPI)) pdl_wait();
     if (a.pdl_trigger_late) pdl_launch_dependents();
     if (TF32 && MODE == TC_DENSE && a.rt_info && warp < TC_NUM_EPI) {
         // fp32 fc1 storing each token's row at its routing slot (as the 2-SM fc1 does): the
@@ -358,6 +366,7 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
             uint32_t issued = 0;  // bit s: stage s has a load in flight or done
             uint32_t par = 0;     // bit s: parity of stage s's last load
             bool ok = true;
+            bool waited = !TF32 || a.pdl_wait_role != 2;  // role 2: wait before the first t-segment load
             for (int unit = blockIdx.x; unit < num_tiles * ksp && ok; unit += gridDim.x) {
                 TileInfo t = decode_tile(a, unit / ksp, n_tiles, s_prefix, BN);
                 t.e = warp_uniform(t.e);
@@ -372,11 +381,15 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
                     const uint32_t sA = smem_u32(sm + stage * C::STAGE_BYTES);
                     const uint32_t sB = sA + C::A_BYTES;
                     mbar_arrive_expect_tx_warp(full_bar(stage), C::LOAD_BYTES);
-                    if (kb < nk0) {
-                        tma_load_2d(sA, &a.tmA0, kb * KE, (int)t.m0, full_bar(stage));
-                        tma_load_2d(sB, &a.tmB0, kb * KE, t.n0, full_bar(stage));
+                    const int kk = seg_block(kb) * KE;
+                    if (in_k0(kb)) {
+                        if (!waited) {
+                            pdl_wait();
+                            waited = true;
+                        }
+                        tma_load_2d(sA, &a.tmA0, kk, (int)t.m0, full_bar(stage));
+                        tma_load_2d(sB, &a.tmB0, kk, t.n0, full_bar(stage));
                     } else {
-                        const int kk = (kb - nk0) * KE;
                         tma_load_2d(sA, &a.tmA1, kk, (int)t.m0, full_bar(stage));
                         tma_load_2d(sB, &a.tmB1[t.e], kk, t.n0, full_bar(stage));
                     }
@@ -525,7 +538,7 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
                     tc_fence_after();
                     const uint64_t da = d0 + (uint64_t)((stage * C::STAGE_BYTES) >> 4);
                     const uint64_t db = da + (uint64_t)(C::A_BYTES >> 4);
-                    const int kvalid = kb < nk0 ? min(KE, a.K0 - kb * KE) : min(KE, a.K1 - (kb - nk0) * KE);
+                    const int kvalid = min(KE, (in_k0(kb) ? a.K0 : a.K1) - seg_block(kb) * KE);
                     if constexpr (TF32) {
                         // K = 8 per MMA (32 bytes = 2 descriptor units); columns past K were filled with
                         // zeros by the TMA
@@ -578,6 +591,8 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
         int acc = 0;
         uint32_t aph = 0;
         uint32_t kph = 0;  // fp32 K split: parity of the handshake barriers
+        // the basis kernel may still use the K-split workspace and counters
+        if (TF32 && a.pdl_wait_role == 2) pdl_wait();
         volatile int* s_last = reinterpret_cast<volatile int*>(tmem_slot + 2);
         for (int unit = blockIdx.x; unit < num_tiles * ksp; unit += gridDim.x) {
             const int tile = unit / ksp;

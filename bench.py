@@ -51,7 +51,8 @@ NOMINAL_PEAKS = {"hbm_gbs": 7900.0, "bf16_tflops": 2250.0}
 TF32X3_OF_BF16 = 1.1 / 2.25 / 3
 STAGES = ("route", "fc1_gelu", "basis", "grouped")
 KERNEL_OF_STAGE = {"route": "cm::route_tc_kernel",
-                   "fc1_gelu": "cm::tc_gemm2_kernel<256, 0, 0> (2-SM dense, rows stored at their routing slots)",
+                   "fc1_gelu": "cm::tc_gemm2_kernel<256, 0, 4> (2-SM dense, bias + GELU, rows stored at their routing slots; "
+                               "<256, 0, 3> at d <= 512)",
                    "basis": "cm::tc_gemm2_kernel<128, 0, 0> (2-SM dense, column scale)",
                    "grouped": "cm::tc_gemm2_kernel<256, 2, 0> (2-SM grouped, rows stored at perm[slot])"}
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) from the committed ncu

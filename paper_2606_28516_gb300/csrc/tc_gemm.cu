@@ -16,7 +16,8 @@
 // Stages of a shared-memory ring are handed over by mbarriers (full: TMA bytes / cp.async
 // arrivals; empty: tcgen05.commit). Two TMEM accumulators let the epilogue of one tile overlap the
 // MMAs of the next. The grouped mode walks tiles (expert, m-tile, n-tile) from the device-resident
-// expert offsets and chains two K segments into one accumulator: [t | z] x [U_r | W_e^res].
+// expert offsets and chains two K segments into one accumulator: [t | z] x [U_r | W_e^res], the fp32
+// variant z's first, which may run beside the basis kernel that forms t.
 // Every wait is bounded; on time-out the CTA records CLEARMOE_ETIMEOUT, drains its in-flight
 // copies and MMAs, frees TMEM and returns.
 //
@@ -35,8 +36,9 @@
 // rows and the K-split partials are stored with consecutive lanes on consecutive bytes (one row per
 // lane touched 32 rows with 16 bytes each), and GELU takes the branch-free form of common.cuh.
 // Measured (DeiT-T layer, whole forwards): T = 12,608: 125 us with both operands in shared memory, 112
-// with coalesced stores, 93 with A in tensor memory, 87.5 with the branch-free GELU; T = 788: 48.1 /
-// 42.5 / 38.8 / 37.1 us. Results differ from the first form's only through GELU.
+// with coalesced stores, 93 with A in tensor memory, 87.5 with the branch-free GELU, 86 with no option tests,
+// 83.9 without the slot kernel (route_grid), 79.6 with the products started beside the previous kernel; T =
+// 788: 48.1 / 42.5 / 38.8 / 37.1 / 34.6 / 34.0 / 30.3 us.
 #include <cstdint>
 #include <mutex>
 

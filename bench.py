@@ -59,10 +59,10 @@ KERNEL_OF_STAGE = {"route": "cm::route_tc_kernel",
 # capture (profiles/clearmoe_kernels_deit_base_T50432_full.md), with the hash of the kernel's sources
 # it was taken on (source_hash); a different hash means the kernel changed and the figure is void.
 TRAFFIC = {
-    "route": {"bytes": 78.52416e6, "src": "3deea90ad96906dc"},
-    "fc1_gelu": {"bytes": 338.377472e6, "src": "eb41af172793f61c"},
-    "basis": {"bytes": 316.010752e6, "src": "eb41af172793f61c"},
-    "grouped": {"bytes": 426.028544e6, "src": "eb41af172793f61c"},
+    "route": {"bytes": 78.3616e6, "src": "08aac3317c96498b"},
+    "fc1_gelu": {"bytes": 338.044416e6, "src": "a6987638f04249d6"},
+    "basis": {"bytes": 315.84e6, "src": "a6987638f04249d6"},
+    "grouped": {"bytes": 426.023168e6, "src": "a6987638f04249d6"},
 }
 
 

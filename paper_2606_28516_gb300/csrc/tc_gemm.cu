@@ -37,8 +37,8 @@
 // lane touched 32 rows with 16 bytes each), and GELU takes the branch-free form of common.cuh.
 // Measured (DeiT-T layer, whole forwards): T = 12,608: 125 us with both operands in shared memory, 112
 // with coalesced stores, 93 with A in tensor memory, 87.5 with the branch-free GELU, 86 with no option tests,
-// 83.9 without the slot kernel (route_grid), 79.6 with the products started beside the previous kernel; T =
-// 788: 48.1 / 42.5 / 38.8 / 37.1 / 34.6 / 34.0 / 30.3 us.
+// 83.9 without the slot kernel (route_grid), 79.5 with the products started beside the previous kernel, 77.0
+// with whole warps staging their rows; T = 788: 48.1 / 42.5 / 38.8 / 37.1 / 34.6 / 34.0 / 30.4 / 30.4 us.
 #include <cstdint>
 #include <mutex>
 
@@ -161,13 +161,36 @@ __device__ __forceinline__ void f32_bias_act(float* f, float4 b, int epi) {
     f[3] = p1.y;
 }
 
-// fp32 rows of a warp (lane = row, CW values each in f) to C through shared memory, half a warp's rows at
-// a time: 16-byte piece j of row rw at piece j ^ (rw & mask), then each store instruction writes
-// 512 contiguous-by-row bytes (CW x 4 bytes per row) where one row per lane would touch 32 rows with 16
-// bytes each. wstg: 16 x CW x 4 bytes of the warp's own.
+// fp32 rows of a warp (lane = row, CW values each in f) to C through shared memory, half a warp's rows
+// (CW = 32: half the columns of all rows) at a time: 16-byte pieces swizzled by row, then each store
+// instruction writes rows of 64 bytes or more (64 in whole sectors at CW = 32) where one row per lane would
+// touch 32 rows with 16 bytes each. At CW = 32 no lane idles and a row's address is formed once for both
+// halves: DeiT-T layer at 12,608 tokens 79.5 -> 77.0 us against half a warp's whole rows at a time. wstg: 16 x
+// CW x 4 bytes of the warp's own.
 template <int CW>
 __device__ __forceinline__ void store_rows_f32(unsigned char* wstg, int lane, const float* f, int64_t orow, float* C,
                                                int64_t ldc, int nb) {
+    if constexpr (CW == 32) {
+        int64_t o[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) o[p] = __shfl_sync(0xffffffffu, orow, 8 * p + (lane >> 2));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                *reinterpret_cast<float4*>(wstg + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) =
+                    make_float4(f[16 * h + 4 * j], f[16 * h + 4 * j + 1], f[16 * h + 4 * j + 2], f[16 * h + 4 * j + 3]);
+            __syncwarp();
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const int rw = 8 * p + (lane >> 2), j = lane & 3;
+                const float4 v = *reinterpret_cast<const float4*>(wstg + rw * 64 + ((j ^ ((rw >> 1) & 3)) << 4));
+                if (o[p] >= 0) *reinterpret_cast<float4*>(C + o[p] * ldc + nb + 16 * h + 4 * j) = v;
+            }
+            __syncwarp();
+        }
+        return;
+    }
     constexpr int LPR = CW / 4;   // lanes (16-byte pieces) per row
     constexpr int RPP = 32 / LPR; // rows per store instruction
 #pragma unroll

@@ -53,33 +53,33 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // GELU of a pair for the bf16 layer, whose hidden state is stored in bf16: GELU(u) = max(u, 0) - |u| / 2
 // erfc(|u| / sqrt 2), with erfc(t / sqrt 2) = 2^q(t) and q a polynomial of degree 6 without constant
 // term, fitted here to log2 erfc(t / sqrt 2) on [0, 5.5] by reweighted least squares in the error it makes
-// in GELU (8.3e-8); t is held at 6, where the second term is 6e-9. Horner's rule runs on v = -t with the
-// odd coefficients' signs turned, and the factor 1/2 is a -1 in the exponent, so that the result is one
-// fma: 7 packed fp32x2 operations and two ex2 a pair. What it costs is fc1's bound in short K and its
-// energy in long: with the rational form of Abramowitz & Stegun 7.1.28 (12 packed operations, two
-// reciprocals, error up to 7.1e-7 in fp32) the ViT-B layer at 50,432 tokens took 401 us under load, now
-// 395, the dense FFN at 100,864 tokens 660 and 644, the 12-sublayer stack at 25,216 tokens 2,420 and 2,361,
-// the DeiT-S layer at 12,608 tokens 49.0 and 47.6.
-// Error against float64: at most 3.2e-7 for every u, mean square below that form's at every width
-// (tests/test_gelu_exp2.py), far below the bf16 spacing of z. NaN gives NaN.
+// in GELU (8.3e-8). Past 5.5 it falls on until t = 14, where t is held and the second term is 2e-35.
+// Horner's rule runs on v = -t with the odd coefficients' signs turned, and the factor 1/2 is a -1 in the
+// exponent, so that the result is one fma: 7 packed fp32x2 operations and two ex2 a pair, and one more for
+// the infinities. What it costs is fc1's bound in short K and its energy in long.
+// Error against float64: at most 3.2e-7 for every u (the rational form of Abramowitz & Stegun 7.1.28 in fp32:
+// 7.1e-7), in every interval below -5 smaller than that form's, and mean square below it at every width
+// (tests/test_gelu_exp2.py). These are absolute bounds: down to u = -4.25 the error is at most a quarter of the
+// bf16 spacing of z; the relative error reaches 0.2 % at -4.5 and 0.5 % at -5 (|z| = 1.4e-6), where half a bf16
+// step is 0.2 to 0.4 %. NaN and -inf give NaN and inf gives inf, as u (1 + erf(u / sqrt 2)) / 2 does.
 struct GeluE {
     static constexpr float C6 = 2.992490044562146e-05f, C5 = 0.0007398800225928426f, C4 = 0.007977480068802834f,
                            C3 = 0.05323820933699608f, C2 = -0.45891568064689636f, C1 = 1.1511471271514893f;
+    static constexpr float HOLD = -14.f;
 };
-__device__ __forceinline__ float relu_nan(float x) {  // max(x, 0), NaN for NaN
-    float y;
-    asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(y) : "f"(x));
-    return y;
-}
 __device__ __forceinline__ float2 gelu_pair_bf16(float2 u) {
-    const float2 v = make_float2(fmaxf(-fabsf(u.x), -6.f), fmaxf(-fabsf(u.y), -6.f));
+    const float2 v = make_float2(fmaxf(-fabsf(u.x), GeluE::HOLD), fmaxf(-fabsf(u.y), GeluE::HOLD));
     float2 q = __ffma2_rn(make_float2(GeluE::C6, GeluE::C6), v, make_float2(GeluE::C5, GeluE::C5));
     q = __ffma2_rn(q, v, make_float2(GeluE::C4, GeluE::C4));
     q = __ffma2_rn(q, v, make_float2(GeluE::C3, GeluE::C3));
     q = __ffma2_rn(q, v, make_float2(GeluE::C2, GeluE::C2));
     q = __ffma2_rn(q, v, make_float2(GeluE::C1, GeluE::C1));
     q = __ffma2_rn(q, v, make_float2(-1.f, -1.f));
-    return __ffma2_rn(v, make_float2(ex2_approx(q.x), ex2_approx(q.y)), make_float2(relu_nan(u.x), relu_nan(u.y)));
+    // max(u, 0) = u / 2 + |u| / 2 exactly, NaN for -inf and NaN (max.NaN(u, 0) would give 0 for -inf, and 46.7 us
+    // against 46.8 for the DeiT-S layer at 12,608 tokens, 85.9 against 86.3 for the dense ViT-B FFN there)
+    const float2 half = make_float2(0.5f, 0.5f);
+    const float2 relu = __ffma2_rn(half, u, make_float2(0.5f * fabsf(u.x), 0.5f * fabsf(u.y)));
+    return __ffma2_rn(v, make_float2(ex2_approx(q.x), ex2_approx(q.y)), relu);
 }
 
 // GELU of a pair in fp32 for the tensor-core fp32 layer: GELU(u) = max(u, 0) - |u| / 2 erfc(|u| / sqrt 2),

@@ -1,13 +1,12 @@
-"""The bf16 layer evaluates GELU with the erf approximation of Abramowitz & Stegun 7.1.28
-(Hastings): erf(x) = 1 - (1 + a1 x + ... + a6 x^6)^-16, |error| <= 3e-7. The kernel writes
+"""The erf approximation of Abramowitz & Stegun 7.1.28 (Hastings), erf(x) = 1 - (1 + a1 x + ... +
+a6 x^6)^-16 with |error| <= 3e-7, in GELU: the form that the bf16 layer evaluated before the one of
+tests/test_gelu_exp2.py, which is held against it there. No kernel has it any more. It wrote
 GELU(u) = max(u, 0) + m y with m = -|u| / 2 and y = P^-16, running Horner's rule on m with the
-coefficients (which carry 1/sqrt(2)^k) scaled by 2^k and alternating in sign, which gives -P. This
-checks, on the CPU with float32 arithmetic in the kernel's order (each fma rounded once from a
-float64 value, where the product is exact), that this form equals plain Horner in |u| bit for bit,
-that the resulting GELU stays within 7.5e-7 of the float64 exact-erf GELU for every u, and that the
-bf16-rounded hidden state it produces differs from the exactly rounded one for a negligible share
-of realistic pre-activations (the rounding of z to bf16 is the layer's declared quantisation
-point)."""
+coefficients (which carry 1/sqrt(2)^k) scaled by 2^k and alternating in sign, which gives -P. These
+checks pin the float32 model down (each fma rounded once from a float64 value, where the product is
+exact): this form equals plain Horner in |u| bit for bit, the resulting GELU stays within 7.5e-7 of
+the float64 exact-erf GELU for every u, and the bf16-rounded hidden state it produced differs from
+the exactly rounded one for a negligible share of realistic pre-activations."""
 import numpy as np
 from scipy.special import erfc
 
@@ -32,7 +31,7 @@ def _poly_plain(au):
 
 
 def _poly_kernel(m):
-    """The kernel's form: Horner on m = -|u| / 2 with c_k = (-1)^(k+1) b_k 2^k; returns -P."""
+    """The former kernel's: Horner on m = -|u| / 2 with c_k = (-1)^(k+1) b_k 2^k; returns -P."""
     c = [np.float32((-1) ** (k + 1) * float(bk) * 2.0 ** k) for k, bk in enumerate(_b())]
     p = _fma32(np.full_like(m, c[6]), m, c[5])
     for k in (4, 3, 2, 1, 0):
@@ -70,7 +69,7 @@ def test_kernel_horner_form_is_exact():
 
 
 def test_relu_as_half_sum_is_exact():
-    """The kernel forms max(u, 0) as the fma u * 0.5 + |u| / 2 (m = -|u| / 2 negated): exact
+    """The form takes max(u, 0) as the fma u * 0.5 + |u| / 2 (m = -|u| / 2 negated): exact
     wherever halving is (|u| >= 2^-125; below that GELU(u) rounds to zero in bf16 anyway)."""
     rng = np.random.default_rng(5)
     u = np.concatenate([rng.standard_normal(500_000) * 10.0 ** rng.integers(-30, 30, 500_000),

@@ -453,6 +453,7 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
                     ok = false;
                     break;
                 }
+                tc_fence_after();  // the stage's earlier MMAs read the tensor memory written below
                 const unsigned char* sA = sm + stage * C::STAGE_BYTES + row * 128;
                 uint32_t h[32], l[32];
 #pragma unroll

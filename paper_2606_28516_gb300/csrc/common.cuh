@@ -178,7 +178,9 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
-// mbar_wait by a whole warp: every lane returns the same outcome.
+// mbar_wait by a whole warp: every lane returns the same outcome. Each lane reads the clock and the abort
+// flag for itself, so near the limit single lanes may give up; what follows a wait is run by the whole warp
+// (tcgen05.ld, shuffles, __syncwarp, elect.sync) and needs all lanes or none.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort, int32_t* status,
                                                uint64_t limit_ns) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, status, limit_ns));

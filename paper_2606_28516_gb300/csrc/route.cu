@@ -239,8 +239,7 @@ __global__ void __launch_bounds__(RTC_THREADS, 1) route_tc_kernel(const __grid_c
             const bool valid = i < nrows;
             const int64_t row = row0 + i;
             const float2 ln = (lnf && valid) ? a.ln_stats[row] : make_float2(0.f, 1.f);
-            // the warp agrees on the outcome, so that its tcgen05.ld runs on all lanes or none
-            const bool ok = __all_sync(0xffffffffu, mbar_wait(tfull_bar(acc), (j >> 1) & 1, abort_flag, a.status, lim));
+            const bool ok = mbar_wait_warp(tfull_bar(acc), (j >> 1) & 1, abort_flag, a.status, lim);
             int esel = -1;  // this lane's expert (E: a class token; -1: no row)
             if (ok) {
                 tc_fence_after();

@@ -625,7 +625,7 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
             const TileInfo t = decode_tile(a, tile, n_tiles, s_prefix, BN);
             int klo = 0, khi = 1;
             if (TF32) k_range(t, unit % ksp, klo, khi);
-            if (!mbar_wait(tfull_bar(acc), aph, abort_flag, a.status, lim)) break;
+            if (!mbar_wait_warp(tfull_bar(acc), aph, abort_flag, a.status, lim)) break;
             tc_fence_after();
             const int r = q * 32 + lane;
             int64_t orow = -1;
@@ -786,10 +786,9 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
                     *s_last = last;
                     mbar_arrive(kdone_bar);
                 }
-                const bool done = mbar_wait(kdone_bar, kph, abort_flag, a.status, lim);
+                const bool done = mbar_wait_warp(kdone_bar, kph, abort_flag, a.status, lim);
                 kph ^= 1;
-                // the warp agrees (a wait that gave up ends it for single lanes), so that its rows are stored together
-                if (__all_sync(0xffffffffu, done && *s_last)) {
+                if (__all_sync(0xffffffffu, done && *s_last)) {  // the warp stores its rows together
                     __threadfence();
                     for (int c = c_lo; c < c_lo + C::HALF; c += C::CW) {
                         float f[C::CW];

@@ -535,7 +535,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
             const uint32_t rtw = (MODE == TC_DENSE && a.rt_info && mrow < t.hi) ? (uint32_t)a.rt_info[mrow] : 0u;
             // the LayerNorm folded into A: (mean, rstd) of this lane's row, loaded early for the same reason
             const float2 ln = (a.ln_stats && mrow < t.hi) ? a.ln_stats[mrow] : make_float2(0.f, 1.f);
-            if (!mbar_wait(tfull_bar(acc), aph, abort_flag, a.status, lim)) break;
+            if (!mbar_wait_warp(tfull_bar(acc), aph, abort_flag, a.status, lim)) break;
             tc_fence_after();
             if (VAR == TC2_ROUTER && t.router) {
                 // The router unit: accumulator columns [0, E) of this lane's row hold W_g x. The four
@@ -574,7 +574,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(fr_bar(rb));
-                    if (mbar_wait(fr_bar(rb), (uint32_t)(fr_it >> 1) & 1u, abort_flag, a.status, lim)) {
+                    if (mbar_wait_warp(fr_bar(rb), (uint32_t)(fr_it >> 1) & 1u, abort_flag, a.status, lim)) {
                         if (esel >= 0) {
                             int base = 0;
                             for (int qq = 0; qq < q; ++qq) base += rc[qq * CM_MAX_E + esel];

@@ -1,7 +1,8 @@
 """Rules that the kernels' waits keep, checked on the sources (a hardware run cannot show that one is broken,
 and must not try): by the PTX memory model a tcgen05 operation is ordered after a barrier wait only by
 tcgen05.fence::after_thread_sync, so that every access to tensor memory (MMA, load, store) follows the last
-barrier wait before it with such a fence in between."""
+barrier wait before it with such a fence in between; and a bounded wait may run out for single lanes of a
+warp, so that a warp takes its outcome together (mbar_wait_warp): what follows is collective over the warp."""
 import pathlib
 import re
 
@@ -30,3 +31,13 @@ def test_tensor_memory_accesses_follow_a_fence(name):
         assert last is not None, m.group()
         line = s[:m.start()].count("\n")
         assert "tc_fence_after();" in s[last:m.start()], f"{name}, line {line} of the kernels: {m.group()}"
+
+
+@pytest.mark.parametrize("name", FILES)
+def test_warps_agree_on_a_wait_that_ran_out(name):
+    s = _source(name)
+    single = re.findall(r"\bmbar_wait\((\w+)", s)
+    # the K split's counter: lane 0 of warp 0 alone
+    assert [b for b in single if b != "kjoin_bar"] == []
+    for m in re.finditer(r"\bmbar_wait\(kjoin_bar", s):
+        assert "if (warp == 0 && lane == 0) {" in s[m.start() - 200:m.start()]

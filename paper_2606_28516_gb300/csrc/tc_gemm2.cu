@@ -18,6 +18,7 @@
 // output row m goes to C[a.rows[m]] (fc1: inv[token] = slot; grouped: perm[slot] = token).
 // Every wait is bounded; both CTAs always reach the closing cluster barrier.
 #include "common.cuh"
+#include "drain.h"
 #include "internal.h"
 
 namespace cm {
@@ -48,8 +49,11 @@ struct T2 {
     static constexpr int STG_BYTES = NUM_EPI * 32 * STG_ROW;
     static constexpr int BIAS_CAP = TC2_BIAS_CAP;         // fp32 bias / scale staged in shared memory
     static constexpr int TAB_CAP = TC2_TAB_CAP;           // routing prefix table (fused fc1)
-    static constexpr int NBARS = 2 * STAGES + 7;  // + 2 for the router inside fc1
+    static constexpr int NBARS = 2 * STAGES + 8;  // 2 of them for the router inside fc1
     static constexpr int FR_B_BYTES = 16 * BK * 2;        // the router unit's B box per CTA: 16 rows of W_g
+    // after the barriers 128 bytes: tensor-memory base, abort flag, 2 unused words, group prefixes, and the
+    // producer's 1 + STAGES words
+    static_assert((4 + CM_MAX_E + 1 + 1 + STAGES) * 4 <= 128);
     static constexpr int SMEM =
         1024 + STAGES * STAGE_BYTES + STG_BYTES + BIAS_CAP * 4 + (TAB_CAP + CM_MAX_E) * 4 + NBARS * 8 + 128;
     static constexpr int TMEM_COLS = 2 * BN <= 256 ? 256 : 512;  // two accumulators (a power of 2)
@@ -129,9 +133,31 @@ __device__ __forceinline__ void umma2_commit_one(uint32_t bar) {  // arrive on t
         "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
         : "memory");
 }
+// Counts `bytes` of a barrier's phase as landed, by the elected lane of a converged warp.
+__device__ __forceinline__ void mbar_complete_tx_warp(uint32_t bar, uint32_t bytes) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;\n\t}" ::"r"(bar), "r"(bytes)
+        : "memory");
+}
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr_cluster) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr_cluster) : "memory");
+    return v;
+}
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
 }
+// By a converged warp's elected lane, whose writes before it the other CTA sees behind its wait and fence_cluster().
+__device__ __forceinline__ void mbar_arrive_release_cluster_warp(uint32_t bar_cluster) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n\t}" ::"r"(bar_cluster)
+        : "memory");
+}
+__device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 
 struct PairTile {
     int64_t m0;  // first row of the pair tile (CTA r starts at m0 + 128 r)
@@ -209,6 +235,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + NBARS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     int* s_prefix = reinterpret_cast<int*>(tmem_slot + 4);  // [CM_MAX_E + 1]
+    // [0] the stages this CTA's producer has issued, once it has stopped; [1 + s] its bytes of stage s's last use
+    volatile uint32_t* s_issued = reinterpret_cast<uint32_t*>(s_prefix + CM_MAX_E + 1);
+    const uint32_t issued_addr = smem_u32(s_prefix + CM_MAX_E + 1);
 
     if (!a.pdl_trigger_late) pdl_launch_dependents();
     const int warp = warp_uniform((int)threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -223,6 +252,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
     // the router inside fc1: the four lane-quarter warps' expert counts of a router unit are
     // exchanged through shared memory, double-buffered, each buffer guarded by its own barrier
     auto fr_bar = [&](int i) { return bar0 + 8u * (2 * STAGES + 5 + i); };
+    const uint32_t stop_bar = bar0 + 8u * (2 * STAGES + 7);  // even CTA: both producers have stopped
     int* s_frc = s_tab;                                            // [2][4][CM_MAX_E] counts
     float* s_frb = reinterpret_cast<float*>(s_tab + 8 * CM_MAX_E);  // [CM_MAX_E] b_g
     const uint64_t lim = (uint64_t)a.wait_limit_ns;
@@ -245,6 +275,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
         mbar_init(drain_bar, 1);
         mbar_init(fr_bar(0), 4);  // the quarter warps of the first column group
         mbar_init(fr_bar(1), 4);
+        mbar_init(stop_bar, 2);
         *abort_flag = 0;
         mbar_fence_init();
     }
@@ -391,7 +422,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
         constexpr bool gather = VAR == TC2_GATHER;
         bool waited = a.pdl_wait_role != 2;  // role 2: wait before the first t-segment load
         int stage = 0;
-        uint32_t ph = 0;
+        uint32_t ph = 0, issued = 0;
         bool ok = true;
         for (int u = cid; u < num_units && ok; u += ncl) {
             PairTile t = decode_pair<BN, VAR>(a, u, full, n_tiles, s_prefix);
@@ -399,7 +430,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
             const int am = warp_uniform((int)(t.m0 + (int64_t)rank * BM));
             // the router unit: CTA r supplies W_g rows [16 r, +16) of the 256 x 32 MMA
             const int bn = t.router ? (int)rank * 16 : t.n0 + (int)rank * (t.half ? BH / 2 : BH);
-            const uint32_t stage_tx = 2u * (A_BYTES + (t.router ? C::FR_B_BYTES : t.half ? C::B_BYTES / 2 : C::B_BYTES));
+            const uint32_t cta_tx = A_BYTES + (t.router ? C::FR_B_BYTES : t.half ? C::B_BYTES / 2 : C::B_BYTES);
             const int nkb_t = (MODE == TC_GROUPED && a.dense_last && t.e == a.E - 1) ? nk1 : nkb;
             int32_t gr[4] = {0, 0, 0, 0};
             if (gather) {  // this lane's four slots; slots past M take the last one (their rows are dropped)
@@ -418,7 +449,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                     const uint32_t sA = smem_u32(sm + stage * STAGE_BYTES);
                     const uint32_t sB = sA + A_BYTES;
                     const uint32_t fb = full_leader0 + 8u * stage;  // the even CTA's full barrier
-                    if (leader) mbar_arrive_expect_tx_warp(full_bar(stage), stage_tx);
+                    if (leader) mbar_arrive_expect_tx_warp(full_bar(stage), 2u * cta_tx);
                     const int kk = kb * BK;
                     if (gathered)
                         tma_gather4_pair(sA + 512u * lane, mA, kk, gr[0], gr[1], gr[2], gr[3], fb);
@@ -427,6 +458,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                     else
                         tma_load_2d_pair(sA, mA, kk, am, fb);
                     tma_load_2d_pair(sB, mB, kk, bn, fb);
+                    s_issued[1 + stage] = cta_tx;
+                    ++issued;
                     if (++stage == STAGES) {
                         stage = 0;
                         ph ^= 1;
@@ -448,6 +481,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
                 }
             }
         }
+        *s_issued = issued;
+        __syncwarp();
+        mbar_arrive_release_cluster_warp(map_to_rank(stop_bar, 0));
     } else if (warp == WARP_MMA) {
         // ------------------------------------------------ MMA issuer (even CTA, the whole warp)
         if (leader) {
@@ -506,6 +542,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
             }
             umma2_commit_one(drain_bar);
             mbar_wait_warp(drain_bar, 0, nullptr, a.status, 10000000ull);
+            // An issuer that ran all its units has seen every copy of both CTAs land. One that gave up waits,
+            // once both producers have stopped (the other CTA's after its own limit), for the last copies issued
+            // to each stage; a stage that only one producer reached gets the other's part of its barrier here.
+            // (Kept small: walking the units for their bytes here cost the DeiT-S layer at 197 tokens 0.4 us of
+            // 21.1, a plain store to the other CTA's shared memory 20 registers and 7 of 47 us at 12,608.)
+            if (warp_uniform((int)*abort_flag) && mbar_wait_warp(stop_bar, 0, nullptr, a.status, 2 * lim + 10000000ull)) {
+                fence_cluster();
+                const uint32_t peer = map_to_rank(issued_addr, 1);
+                const uint32_t n0 = ld_cluster_u32(map_to_rank(issued_addr, 0)), n1 = ld_cluster_u32(peer), n = max(n0, n1);
+#pragma unroll 1
+                for (uint32_t k = n > STAGES ? n - STAGES : 0; k < n; ++k) {
+                    const uint32_t s = k % STAGES;
+                    const DrainStep d = drain_step(k, n0, n1);
+                    if (d.arrive) mbar_arrive_expect_tx_warp(full_bar(s), ld_cluster_u32(peer + 4 * (1 + s)));
+                    if (d.complete) mbar_complete_tx_warp(full_bar(s), s_issued[1 + s]);
+                    mbar_wait_warp(full_bar(s), (k / STAGES) & 1, nullptr, a.status, 10000000ull);
+                }
+            }
         }
         __syncwarp();
     } else if (warp < NUM_EPI) {

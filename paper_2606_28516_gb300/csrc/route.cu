@@ -181,10 +181,11 @@ __global__ void __launch_bounds__(RTC_THREADS, 1) route_tc_kernel(const __grid_c
                     tma_load_3d(dst + (uint32_t)b * box_bytes, &A.tmX, 0, r + b * RTC_BOX_ROWS, h * nkc, full_bar(s));
             }
         }
-        if (!ok)  // gave up: let the copies in flight land before the CTA moves on
-            for (int j = max(0, k - S); j < k; ++j)
-                mbar_wait_warp(full_bar(j % S), (j / S) & 1, nullptr, a.status, 10000000ull);
-        if (nblk > 0) mbar_wait_warp(wbar, 0, nullptr, a.status, 10000000ull);  // W_g's boxes have landed too
+        // the copies in flight land before the CTA moves on, whoever gave up (the issuer may after the last is
+        // issued), W_g's boxes too
+        for (int j = max(0, k - S); j < k; ++j)
+            mbar_wait_warp(full_bar(j % S), (j / S) & 1, nullptr, a.status, lim + 10000000ull);
+        if (nblk > 0) mbar_wait_warp(wbar, 0, nullptr, a.status, lim + 10000000ull);
     } else if (issuer) {
         const uint32_t idesc = idesc_bf16_f32(RTC_BM, 16);
         // a K block's descriptor is the ring base's plus the byte offset / 16 (addresses stay below

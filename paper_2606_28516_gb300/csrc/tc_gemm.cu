@@ -426,10 +426,10 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
                     }
                 }
             }
-            if (!ok) {  // let every copy in flight land before the CTA retires
-                for (int s = 0; s < C::STAGES; ++s)
-                    if (issued & (1u << s)) mbar_wait_warp(full_bar(s), (par >> s) & 1, nullptr, a.status, 10000000ull);
-            }
+            // let every copy in flight land before the CTA retires, whoever gave up: the issuer may after this
+            // warp has issued its last
+            for (int s = 0; s < C::STAGES; ++s)
+                if (issued & (1u << s)) mbar_wait_warp(full_bar(s), (par >> s) & 1, nullptr, a.status, lim + 10000000ull);
         }
     } else if (TF32 && warp >= TC_WARP_GATHER) {
         // ------------------------------------------------ fp32: split each landed stage
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
         const int rsub = pt >> 3; // rows rsub + 16 i
         const uint16_t* X = static_cast<const uint16_t*>(a.gather_src);
         int stage = 0;
-        uint32_t ph = 0;
+        uint32_t ph = 0, issued = 0;
         bool ok = true;
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
             const TileInfo t = decode_tile(a, tile, n_tiles, s_prefix, BN);
@@ -527,6 +527,7 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
                 }
                 asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(full_bar(stage))
                              : "memory");
+                ++issued;
                 if (++stage == C::STAGES) {
                     stage = 0;
                     ph ^= 1;
@@ -534,6 +535,17 @@ __global__ void __launch_bounds__(tc_threads<MODE, TF32>(), 1)
             }
         }
         cp_async_wait<0>();
+        // The first warp waits for B's last boxes to land, as the TMA producer does. A wait that ran out stops the
+        // four warps at different stages: the others arrive for the stages of the first that they did not
+        // reach. (s_prefix is the grouped mode's.)
+        volatile int* s_issued = s_prefix;
+        s_issued[warp - TC_WARP_GATHER] = (int)issued;
+        asm volatile("bar.sync 2, %0;" ::"n"(TC_GATHER_THREADS) : "memory");
+        const uint32_t n = (uint32_t)s_issued[0];
+        for (uint32_t k = issued; k < n; ++k) mbar_arrive(full_bar((int)(k % C::STAGES)));
+        if (pt < 32)
+            for (uint32_t k = n > C::STAGES ? n - C::STAGES : 0; k < n; ++k)
+                mbar_wait_warp(full_bar((int)(k % C::STAGES)), (k / C::STAGES) & 1, nullptr, a.status, lim + 10000000ull);
     } else if (warp == TC_WARP_MMA) {
         // ------------------------------------------------ MMA issuer (the whole warp)
         {

@@ -38,6 +38,9 @@ def _call(kind, T, d, H, E, r, dtype):
     ("dense", 300, 256, 32768, 1, 64, "bf16"), ("dense", 3000, 768, 16384, 1, 64, "bf16"),
     ("layer", 9973, 768, 4096, 8, 256, "bf16"), ("layer", 300, 768, 4096, 4, 48, "bf16"),
     ("classes", 6304, 768, 4096, 4, 128, "bf16"), ("router_in_fc1", 3000, 768, 4096, 4, 64, "bf16"),
+    # fc1 on the 1-SM kernel, its rows gathered by slot; the 1-SM kernel throughout; fp32
+    ("layer", 3000, 1024, 8192, 4, 64, "bf16"), ("layer", 1000, 64, 16448, 2, 16, "bf16"),
+    ("layer", 3000, 192, 16384, 4, 32, "f32"), ("dense", 300, 512, 8192, 1, 32, "f32"),
 ])
 def test_gives_up_and_recovers(kind, T, d, H, E, r, dtype):
     h, out, call = _call(kind, T, d, H, E, r, dtype)

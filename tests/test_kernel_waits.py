@@ -41,3 +41,12 @@ def test_warps_agree_on_a_wait_that_ran_out(name):
     assert [b for b in single if b != "kjoin_bar"] == []
     for m in re.finditer(r"\bmbar_wait\(kjoin_bar", s):
         assert "if (warp == 0 && lane == 0) {" in s[m.start() - 200:m.start()]
+
+
+@pytest.mark.parametrize("name", ("route.cu", "tc_gemm.cu"))
+def test_producers_wait_for_their_last_copies_whoever_gave_up(name):
+    # the issuer can give up on a copy in flight after its producer has issued the last one without a wait that
+    # ran out, so that the producer's own outcome does not decide whether copies are in flight
+    s = _source(name)
+    assert not re.search(r"if \(!ok[^)]*\)\s*\{?\s*for \(", s)
+    assert "lim + 10000000ull" in s

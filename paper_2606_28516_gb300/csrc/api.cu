@@ -340,8 +340,11 @@ int clearmoe_layer_create(const clearmoe_layer_desc* desc, clearmoe_layer** out)
                 cudaMalloc((void**)&L->simt_cnt, (size_t)cm::simt_cnt_len(L->num_sms) * 4) == cudaSuccess &&
                 cudaMemset(L->simt_cnt, 0, (size_t)cm::simt_cnt_len(L->num_sms) * 4) == cudaSuccess));
     if (ok) {
-        // index workspaces start at zero (valid rows), so no launch ever reads garbage indices
-        ok = cudaMemset(L->status, 0, 4) == cudaSuccess && cudaMemset(L->perm, 0, T * 4) == cudaSuccess &&
+        // index workspaces and histograms start at zero (valid rows and counts), so no launch ever reads garbage,
+        // also after one that gave up before it had written them
+        ok = cudaMemset(L->cta_counts, 0, ncta * CM_MAX_E * 4) == cudaSuccess &&
+             cudaMemset(L->counts, 0, CM_MAX_E * 4) == cudaSuccess &&
+             cudaMemset(L->offsets, 0, (CM_MAX_E + 1) * 4) == cudaSuccess && cudaMemset(L->status, 0, 4) == cudaSuccess && cudaMemset(L->perm, 0, T * 4) == cudaSuccess &&
              cudaMemset(L->inv, 0, T * 4) == cudaSuccess && cudaMemset(L->tinfo, 0, T * 4) == cudaSuccess &&
              cudaMemset(L->idx, 0, T * 4) == cudaSuccess &&
              cudaDeviceSynchronize() == cudaSuccess;

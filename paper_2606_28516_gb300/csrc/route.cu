@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(256) route_finalize_kernel(const RouteArgs a, 
         const int e = (int)(w & 0xffu);
         if (e >= E) continue;  // only a routing launch that gave up leaves such words
         const int64_t slot = (int64_t)s_base[e] + (int)(w >> 8);
-        if (slot >= a.T) continue;
+        if ((uint64_t)slot >= (uint64_t)a.T) continue;
         a.perm[slot] = (int32_t)(row0 + i);
         if (a.inv) a.inv[row0 + i] = (int32_t)slot;
         if (unpack) a.idx[row0 + i] = e;

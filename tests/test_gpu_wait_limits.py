@@ -65,3 +65,24 @@ def test_gives_up_and_recovers(kind, T, d, H, E, r, dtype):
         assert gave_up[0]
     finally:
         cm.clearmoe_layer_destroy(h)
+
+
+@pytest.mark.parametrize("kind", ["layer", "classes", "router_in_fc1"])
+def test_first_call_gives_up(kind):
+    """A handle whose first calls give up has no routing of an earlier call behind it."""
+    args = (kind, 3000, 768, 4096, 4, 64, "bf16")
+    h, want, call = _call(*args)
+    h2, out, call2 = _call(*args)
+    try:
+        call()
+        assert cm.clearmoe_layer_status(h) == 0
+        cm.clearmoe_debug_set_wait(h2, 1_000, 0)
+        for _ in range(3):
+            call2()
+        assert cm.clearmoe_layer_status(h2) == cm.ETIMEOUT
+        cm.clearmoe_debug_set_wait(h2, 1_000_000_000, 0)
+        call2()
+        assert cm.clearmoe_layer_status(h2) == 0 and torch.equal(out, want)
+    finally:
+        cm.clearmoe_layer_destroy(h)
+        cm.clearmoe_layer_destroy(h2)

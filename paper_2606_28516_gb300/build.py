@@ -38,7 +38,7 @@ def _compile(src: pathlib.Path, verbose: bool) -> pathlib.Path:
 
 def build(verbose: bool = False, force: bool = False) -> pathlib.Path:
     srcs = [CSRC / s for s in SOURCES]
-    deps = srcs + [CSRC / "common.cuh", CSRC / "internal.h", CSRC / "drain.h", PKG.parent / "include" / "clearmoe.h"]
+    deps = srcs + [CSRC / "common.cuh", CSRC / "internal.h", CSRC / "drain.h", CSRC / "tmap_cache.h", PKG.parent / "include" / "clearmoe.h"]
     if OUT.exists() and not force and all(OUT.stat().st_mtime >= p.stat().st_mtime for p in deps):
         return OUT
     BUILD.mkdir(exist_ok=True)

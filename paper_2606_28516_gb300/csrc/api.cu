@@ -45,11 +45,12 @@ namespace {
 using cm::encode_tmap_bf16;
 using cm::encode_tmap_f32;
 
-// A GEMM's B matrix: for the 2-SM kernel at tile width p in boxes of p / 2 rows, and of half as many for
-// its half tiles; for the 1-SM kernel (p = 0) in boxes of bn rows.
-int encode_b_bf16(CUtensorMap* full, CUtensorMap* half, const void* base, int64_t rows, int64_t cols, int p, int bn) {
+// A GEMM's B matrix: for the 2-SM kernel at tile width p in boxes of p / 2 rows and, if the launch may run half
+// tiles (g.half_pairs), of half as many in `half`; for the 1-SM kernel (p = 0) in boxes of bn rows.
+int encode_b_bf16(const cm::TcGemmArgs& g, CUtensorMap* full, CUtensorMap* half, const void* base, int64_t rows,
+                  int64_t cols, int p, int bn) {
     const int rc = encode_tmap_bf16(full, base, rows, cols, p ? p / 2 : bn);
-    return rc || !p ? rc : encode_tmap_bf16(half, base, rows, cols, p / 4);
+    return rc || !p || g.half_pairs <= 0 ? rc : encode_tmap_bf16(half, base, rows, cols, p / 4);
 }
 
 inline bool misaligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
@@ -132,7 +133,8 @@ int mlp_hidden(clearmoe_layer* L, const void* x, int64_t T, const clearmoe_mlp_r
     const int p = nh <= cm::TC2_BIAS_CAP ? cm::tc2_pick_bn(cm::TC_DENSE, nh) : 0;
     const int bn = cm::tc_pick_bn(cm::TC_DENSE, nh);
     if (!p && !bn) return CLEARMOE_EUNSUPPORTED;
-    if (encode_tmap_bf16(&g.tmA0, x, T, d, 128) || encode_b_bf16(&g.tmB0, &g.tmB0h, m->W_in, nh, d, p, bn))
+    g.half_pairs = cm::tc2_dense_half_pairs(T, nh, p, L->num_sms);
+    if (encode_tmap_bf16(&g.tmA0, x, T, d, 128) || encode_b_bf16(g, &g.tmB0, &g.tmB0h, m->W_in, nh, d, p, bn))
         return CLEARMOE_ECUDA;
     g.mode = cm::TC_DENSE;
     g.epi = m->act == CLEARMOE_ACT_GELU ? cm::TC_EPI_BIAS_GELU : cm::TC_EPI_BIAS_RELU;
@@ -201,7 +203,7 @@ int ln_fc1_aug(clearmoe_layer* L, cm::TcGemmArgs& g, int64_t T, int p) {
     g.ln_colsum = nullptr;
     g.ln_aug = 1;
     if (encode_tmap_bf16(&g.tmA1, L->ln_aug_x, T, cm::LN_AUG_K, 128) ||
-        encode_b_bf16(&g.tmB1[0], &g.tmB1h[0], L->ln_aug_w, L->desc.hidden, cm::LN_AUG_K, p, 0))
+        encode_b_bf16(g, &g.tmB1[0], &g.tmB1h[0], L->ln_aug_w, L->desc.hidden, cm::LN_AUG_K, p, 0))
         return CLEARMOE_ECUDA;
     return CLEARMOE_OK;
 }
@@ -459,7 +461,8 @@ static int ffn_router_in_fc1(clearmoe_layer* L, const void* x, int64_t T, const 
         std::memset(&g2, 0, sizeof(g2));
         g2.status = L->status;
         g2.wait_limit_ns = L->wait_limit_ns;
-        if (encode_tmap_bf16(&g2.tmA0, L->z, T, H, 128) || encode_b_bf16(&g2.tmB0, &g2.tmB0h, Vh_r, r, H, p2, bn2))
+        g2.half_pairs = cm::tc2_dense_half_pairs(T, r, p2, L->num_sms);
+        if (encode_tmap_bf16(&g2.tmA0, L->z, T, H, 128) || encode_b_bf16(g2, &g2.tmB0, &g2.tmB0h, Vh_r, r, H, p2, bn2))
             return CLEARMOE_ECUDA;
         g2.mode = cm::TC_DENSE;
         g2.epi = cm::TC_EPI_SCALE;
@@ -751,7 +754,8 @@ static int ffn_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W1,
         g.ln_colsum = L->ln_sums;
     }
     if (p1) {
-        if (encode_tmap_bf16(&g.tmA0, x, T, d, 128) || encode_b_bf16(&g.tmB0, &g.tmB0h, W1, H, d, p1, 0))
+        g.half_pairs = cm::tc2_dense_half_pairs(T, H, p1, L->num_sms);
+        if (encode_tmap_bf16(&g.tmA0, x, T, d, 128) || encode_b_bf16(g, &g.tmB0, &g.tmB0h, W1, H, d, p1, 0))
             return CLEARMOE_ECUDA;
         if (ln && (rc = ln_fc1_aug(L, g, T, p1))) return rc;
         g.mode = cm::TC_DENSE;
@@ -790,8 +794,9 @@ static int ffn_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W1,
         g2.status = L->status;
         g2.wait_limit_ns = L->wait_limit_ns;
         const int p2 = cm::tc2_pick_bn(cm::TC_DENSE, r);
+        g2.half_pairs = cm::tc2_dense_half_pairs(T - n_cls, r, p2, L->num_sms);
         if (encode_tmap_bf16(&g2.tmA0, L->z, T, H, 128) ||
-            encode_b_bf16(&g2.tmB0, &g2.tmB0h, Vh_r, r, H, p2, bn2))
+            encode_b_bf16(g2, &g2.tmB0, &g2.tmB0h, Vh_r, r, H, p2, bn2))
             return CLEARMOE_ECUDA;
         g2.mode = cm::TC_DENSE;
         g2.epi = cm::TC_EPI_SCALE;
@@ -814,18 +819,6 @@ static int ffn_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W1,
     g3.wait_limit_ns = L->wait_limit_ns;
     const int p3 = cm::tc2_grouped_bn(T, d, G, factored ? (T - n_cls + 255) / 256 : 0, L->num_sms);
     g3.bn = p3;
-    if ((factored && (encode_tmap_bf16(&g3.tmA0, L->t, T, r, 128) || encode_b_bf16(&g3.tmB0, &g3.tmB0h, U_r, d, r, p3, bn3))) ||
-        (materialized &&
-         (encode_tmap_bf16(&g3.tmA0, L->z, T, H, 128) || encode_b_bf16(&g3.tmB0, &g3.tmB0h, W_sh, d, H, p3, bn3))) ||
-        encode_tmap_bf16(&g3.tmA1, L->z, T, H, 128))
-        return CLEARMOE_ECUDA;
-    for (int e = 0; e < E; ++e)
-        if (encode_b_bf16(&g3.tmB1[e], &g3.tmB1h[e], residual_e[e], d, H, p3, bn3)) return CLEARMOE_ECUDA;
-    if (n_cls > 0) {  // the dense path's group: W2
-        if (encode_b_bf16(&g3.tmB1[E], &g3.tmB1h[E], opt->W2, d, H, p3, bn3)) return CLEARMOE_ECUDA;
-        g3.dense_last = 1;
-    }
-    g3.out_bias = b2;
     // right after the basis kernel (which releases it only once fc1 has completed) the grouped GEMM
     // starts its z segments at once, on the SMs the basis leaves idle, and waits for the basis only
     // before its first t segment; with no routed rows no basis kernel runs, and fc1 (which releases
@@ -835,6 +828,18 @@ static int ffn_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W1,
         g3.pdl_wait_role = 2;
         g3.half_pairs -= (int)((T - n_cls + 255) / 256 % (L->num_sms / 2));  // the basis kernel's last round
     }
+    if ((factored && (encode_tmap_bf16(&g3.tmA0, L->t, T, r, 128) || encode_b_bf16(g3, &g3.tmB0, &g3.tmB0h, U_r, d, r, p3, bn3))) ||
+        (materialized &&
+         (encode_tmap_bf16(&g3.tmA0, L->z, T, H, 128) || encode_b_bf16(g3, &g3.tmB0, &g3.tmB0h, W_sh, d, H, p3, bn3))) ||
+        encode_tmap_bf16(&g3.tmA1, L->z, T, H, 128))
+        return CLEARMOE_ECUDA;
+    for (int e = 0; e < E; ++e)
+        if (encode_b_bf16(g3, &g3.tmB1[e], &g3.tmB1h[e], residual_e[e], d, H, p3, bn3)) return CLEARMOE_ECUDA;
+    if (n_cls > 0) {  // the dense path's group: W2
+        if (encode_b_bf16(g3, &g3.tmB1[E], &g3.tmB1h[E], opt->W2, d, H, p3, bn3)) return CLEARMOE_ECUDA;
+        g3.dense_last = 1;
+    }
+    g3.out_bias = b2;
     g3.mode = cm::TC_GROUPED;
     g3.epi = cm::TC_EPI_SCATTER;
     g3.M = T;
@@ -1000,7 +1005,8 @@ int clearmoe_ffn_forward_scaled(clearmoe_layer* L, const void* x, int64_t T, con
         std::memset(&g, 0, sizeof(g));
         g.status = L->status;
         g.wait_limit_ns = L->wait_limit_ns;
-        if (encode_tmap_bf16(&g.tmA0, x, T, d, 128) || encode_b_bf16(&g.tmB0, &g.tmB0h, W1, H, d, p1, b1n))
+        g.half_pairs = cm::tc2_dense_half_pairs(T, H, p1, L->num_sms);
+        if (encode_tmap_bf16(&g.tmA0, x, T, d, 128) || encode_b_bf16(g, &g.tmB0, &g.tmB0h, W1, H, d, p1, b1n))
             return CLEARMOE_ECUDA;
         g.mode = cm::TC_DENSE;
         g.epi = cm::TC_EPI_BIAS_GELU;
@@ -1019,7 +1025,8 @@ int clearmoe_ffn_forward_scaled(clearmoe_layer* L, const void* x, int64_t T, con
         std::memset(&g2, 0, sizeof(g2));
         g2.status = L->status;
         g2.wait_limit_ns = L->wait_limit_ns;
-        if (encode_tmap_bf16(&g2.tmA0, L->z, T, H, 128) || encode_b_bf16(&g2.tmB0, &g2.tmB0h, Vh_r, r, H, p2, b2n))
+        g2.half_pairs = cm::tc2_dense_half_pairs(T, r, p2, L->num_sms);
+        if (encode_tmap_bf16(&g2.tmA0, L->z, T, H, 128) || encode_b_bf16(g2, &g2.tmB0, &g2.tmB0h, Vh_r, r, H, p2, b2n))
             return CLEARMOE_ECUDA;
         g2.mode = cm::TC_DENSE;
         g2.epi = cm::TC_EPI_SCALE;
@@ -1041,8 +1048,9 @@ int clearmoe_ffn_forward_scaled(clearmoe_layer* L, const void* x, int64_t T, con
         std::memset(&g3, 0, sizeof(g3));
         g3.status = L->status;
         g3.wait_limit_ns = L->wait_limit_ns;
-        if (encode_tmap_bf16(&g3.tmA0, L->t, T, r, 128) || encode_b_bf16(&g3.tmB0, &g3.tmB0h, U_r, d, r, p3, b3n) ||
-            encode_tmap_bf16(&g3.tmA1, L->z, T, H, 128) || encode_b_bf16(&g3.tmB1[0], &g3.tmB1h[0], R, d, H, p3, b3n))
+        g3.half_pairs = L->num_sms / 2;
+        if (encode_tmap_bf16(&g3.tmA0, L->t, T, r, 128) || encode_b_bf16(g3, &g3.tmB0, &g3.tmB0h, U_r, d, r, p3, b3n) ||
+            encode_tmap_bf16(&g3.tmA1, L->z, T, H, 128) || encode_b_bf16(g3, &g3.tmB1[0], &g3.tmB1h[0], R, d, H, p3, b3n))
             return CLEARMOE_ECUDA;
         g3.bn = p3;
         g3.mode = cm::TC_GROUPED;  // one group over all tokens (no offsets): [z | t'] x [R | U_r]
@@ -1197,7 +1205,8 @@ static int dense_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W
     g.wait_limit_ns = L->wait_limit_ns;
     const int pair1 = H <= cm::TC2_BIAS_CAP ? cm::tc2_fc1_bn(T, H, d, false, L->num_sms) : 0;  // 2-SM tile widths
     const int pair2 = cm::tc2_grouped_bn(T, d, 1, 0, L->num_sms);
-    if (encode_tmap_bf16(&g.tmA0, x, T, d, 128) || encode_b_bf16(&g.tmB0, &g.tmB0h, W1, H, d, pair1, bn1))
+    g.half_pairs = cm::tc2_dense_half_pairs(T, H, pair1, L->num_sms);
+    if (encode_tmap_bf16(&g.tmA0, x, T, d, 128) || encode_b_bf16(g, &g.tmB0, &g.tmB0h, W1, H, d, pair1, bn1))
         return CLEARMOE_ECUDA;
     g.mode = cm::TC_DENSE;
     g.epi = cm::TC_EPI_BIAS_GELU;
@@ -1219,7 +1228,8 @@ static int dense_impl(clearmoe_layer* L, const void* x, int64_t T, const void* W
     std::memset(&g2, 0, sizeof(g2));
     g2.status = L->status;
     g2.wait_limit_ns = L->wait_limit_ns;
-    if (encode_tmap_bf16(&g2.tmA0, L->z, T, H, 128) || encode_b_bf16(&g2.tmB0, &g2.tmB0h, W2, d, H, pair2, bn2))
+    g2.half_pairs = cm::tc2_dense_half_pairs(T, d, pair2, L->num_sms);
+    if (encode_tmap_bf16(&g2.tmA0, L->z, T, H, 128) || encode_b_bf16(g2, &g2.tmB0, &g2.tmB0h, W2, d, H, pair2, bn2))
         return CLEARMOE_ECUDA;
     g2.bn = pair2;
     g2.mode = cm::TC_DENSE;

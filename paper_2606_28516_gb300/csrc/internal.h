@@ -219,8 +219,9 @@ struct TcGemmArgs {
     const int32_t* a1_rows;
     // 2-SM kernel: the pair tile's width (256, 192 or 128, dividing N); 0: tc2_pick_bn(mode, N)
     int bn;
-    // 2-SM kernel: SM pairs that may run half tiles in the last round
-    int half_pairs;  // <= 0: all
+    // 2-SM kernel: SM pairs that may run half tiles in the last round (0: no half tiles, and tmB0h, tmB1h are not
+    // read)
+    int half_pairs;
     // 2-SM dense mode at 256-wide tiles: 12 epilogue warps (three per TMEM lane quarter) and a 160 KB
     // operand ring instead of 8 warps and 192 KB, for short K where the epilogue bounds a tile
     int epi12;
@@ -280,6 +281,13 @@ int tc2_pick_bn(int mode, int N);
 // the basis kernel beside it. tc2_pick_bn's or a narrower one; every width gives the same bits.
 int tc2_fc1_bn(int64_t T, int H, int d, bool slots, int num_sms);
 int tc2_grouped_bn(int64_t T, int d, int G, int64_t basis_pairs, int num_sms);
+// Pair tiles of the last round that run as halves, of `tiles` on `ncl` SM pairs (half_pairs of which may take one).
+__host__ __device__ inline int tc2_tail(int64_t tiles, int ncl, int half_pairs) {
+    const int tail = (int)(tiles % ncl);
+    return 2 * tail <= (ncl < half_pairs ? ncl : half_pairs) ? tail : 0;
+}
+// A dense launch of [T x ..] x [N x ..] at tile width bn: half_pairs, 0 when its last round has no half tiles.
+int tc2_dense_half_pairs(int64_t T, int N, int bn, int num_sms);
 cudaError_t launch_tc_gemm2(const TcGemmArgs& a, int num_sms, cudaStream_t s);
 cudaError_t launch_tc_gemm(const TcGemmArgs& a, int num_sms, cudaStream_t s);
 

@@ -44,6 +44,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "tmap_cache.h"
 
 namespace cm {
 
@@ -1005,20 +1006,8 @@ typedef CUresult (*PFN_encodeTiled_t)(CUtensorMap*, CUtensorMapDataType, cuuint3
                                       const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                       CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Encoded maps are cached by (base, rows, cols, box rows, box chunks), which determine them
-// entirely: a forward encodes up to ~20 maps, and the driver call costs microseconds each on the host.
 namespace {
-struct TmapEntry {
-    const void* base;
-    int64_t rows, cols;
-    int box_rows, box_chunks, elem;
-    bool valid;
-    CUtensorMap map;
-};
-constexpr int TMAP_CACHE = 64;
-TmapEntry g_tmaps[TMAP_CACHE];
-int g_tmap_next = 0;
-std::mutex g_tmap_mu;
+TmapCache<CUtensorMap> g_tmaps;
 }  // namespace
 
 static int encode_tmap_uncached(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows,
@@ -1026,22 +1015,9 @@ static int encode_tmap_uncached(CUtensorMap* map, const void* base, int64_t rows
 
 static int encode_tmap_cached(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows,
                               int box_chunks, int elem) {
-    std::lock_guard<std::mutex> lock(g_tmap_mu);
-    for (int i = 0; i < TMAP_CACHE; ++i) {
-        const TmapEntry& c = g_tmaps[i];
-        if (c.valid && c.base == base && c.rows == rows && c.cols == cols && c.box_rows == box_rows &&
-            c.box_chunks == box_chunks && c.elem == elem) {
-            *map = c.map;
-            return 0;
-        }
-    }
-    const int rc = encode_tmap_uncached(map, base, rows, cols, box_rows, box_chunks, elem);
-    if (rc == 0) {
-        TmapEntry& c = g_tmaps[g_tmap_next];
-        c = TmapEntry{base, rows, cols, box_rows, box_chunks, elem, true, *map};
-        g_tmap_next = (g_tmap_next + 1) % TMAP_CACHE;
-    }
-    return rc;
+    return g_tmaps.get(map, TmapKey{base, rows, cols, box_rows, box_chunks, elem}, [&](CUtensorMap* m) {
+        return encode_tmap_uncached(m, base, rows, cols, box_rows, box_chunks, elem);
+    });
 }
 
 int encode_tmap_bf16(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int box_rows) {

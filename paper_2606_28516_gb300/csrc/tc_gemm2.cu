@@ -402,14 +402,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(T2v<BN_, VAR>::THREA
         m_pairs = (int)((a.M + 2 * BM - 1) / (2 * BM));
     const int cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;
     // Pair tiles, and how many run whole: a last round that would leave more than half of the SM pairs
-    // idle (or a launch with few tiles) runs in half tiles, which take little more than half the time.
+    // idle runs in half tiles, which take little more than half the time. (A dense launch starts no more
+    // pairs than it has tiles, so that with one round or less every tile is whole; a grouped launch does not
+    // know its tiles, and may start more.)
     // half_pairs: beside the basis kernel, only the pairs that start early may take one. Measured
     // (us): DeiT-S layer with Zipf experts, 9,973 tokens (234 and 86 tiles on 76 pairs) 57.7 -> 53.5; stack of
     // 12 ViT-B sublayers, 25,216 tokens (309 tiles of each expert GEMM) 2,513 -> 2,488; dense ViT-B FFN, 788
     // tokens 20.3 -> 19.6. Without the limit a ViT-B layer with class tokens (171 tiles, 50 pairs of
     // basis) went from 129 to 132.
     const int num_tiles = warp_uniform(tmem_ok ? m_pairs * units_per_pair<VAR>(n_tiles) : 0);
-    const int tail = VAR != TC2_ROUTER && VAR != TC2_GATHER && 2 * (num_tiles % ncl) <= min(ncl, a.half_pairs) ? num_tiles % ncl : 0;
+    const int tail = VAR != TC2_ROUTER && VAR != TC2_GATHER && a.half_pairs > 0 ? tc2_tail(num_tiles, ncl, a.half_pairs) : 0;
     const int full = num_tiles - tail, num_units = full + 2 * tail;
 
     if (warp == WARP_TMA) {
@@ -868,9 +870,14 @@ int tc2_grouped_bn(int64_t T, int d, int G, int64_t basis_pairs, int num_sms) {
     return basis_pairs > 0 && rounds >= 1 && rounds <= 2 && over > 0 && 5 * over <= pairs ? next : bn;
 }
 
+int tc2_dense_half_pairs(int64_t T, int N, int bn, int num_sms) {
+    const int64_t tiles = bn ? (T + 255) / 256 * (N / bn) : 0;
+    const int pairs = num_sms / 2, ncl = (int)(tiles < pairs ? tiles : pairs);
+    return ncl > 0 && tc2_tail(tiles, ncl, pairs) > 0 ? pairs : 0;
+}
+
 template <int BN, int MODE, int VAR>
-static cudaError_t launch2(TcGemmArgs a, int num_sms, cudaStream_t s) {
-    if (a.half_pairs <= 0) a.half_pairs = num_sms / 2;
+static cudaError_t launch2(const TcGemmArgs& a, int num_sms, cudaStream_t s) {
     using C = T2v<BN, VAR>;
     const void* fn = (const void*)tc_gemm2_kernel<BN, MODE, VAR>;
     const cudaError_t e = smem_attr_once(fn, C::SMEM);

@@ -997,7 +997,8 @@ int clearmoe_ffn_forward_scaled(clearmoe_layer* L, const void* x, int64_t T, con
         rc = launch_simt(L, g, s);
     } else {
         const int p1 = H <= cm::TC2_BIAS_CAP ? cm::tc2_fc1_bn(T, H, d, false, L->num_sms) : 0;
-        const int p2 = cm::tc2_pick_bn(cm::TC_DENSE, r), p3 = cm::tc2_grouped_bn(T, d, 1, (T + 255) / 256, L->num_sms);
+        const int p2 = cm::tc2_pick_bn(cm::TC_DENSE, r);
+        const int p3 = cm::tc2_grouped_bn(T, d, 1, 0, L->num_sms);  // the basis kernel does not run beside it
         const int b1n = cm::tc_pick_bn(cm::TC_DENSE, H), b2n = cm::tc_pick_bn(cm::TC_DENSE, r);
         const int b3n = cm::tc_pick_bn(cm::TC_GROUPED, d);
         if ((!p1 && !b1n) || (!p2 && !b2n) || (!p3 && !b3n)) return CLEARMOE_EUNSUPPORTED;

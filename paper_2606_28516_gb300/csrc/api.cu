@@ -214,7 +214,8 @@ int do_route(clearmoe_layer* L, const void* x, int64_t T, const clearmoe_router*
     const int rd = mlp ? mlp->hidden : L->desc.d;
     const int rdtype = mlp ? CLEARMOE_F32 : L->desc.dtype;
     int grid = 0, chunk = 0;
-    const int g = cm::route_grid(T, rd, E, rdtype, L->num_sms, &grid, &chunk);
+    const bool w_bf16 = mlp && L->desc.dtype == CLEARMOE_BF16;
+    const int g = cm::route_grid(T, rd, E, rdtype, L->num_sms, &grid, &chunk, w_bf16);
     if (g) return g == -2 ? CLEARMOE_EUNSUPPORTED : CLEARMOE_ECUDA;
     if (grid > cm::route_max_ctas(L->num_sms, rdtype, rd, E)) return CLEARMOE_EUNSUPPORTED;
     if (mlp) {
@@ -230,7 +231,7 @@ int do_route(clearmoe_layer* L, const void* x, int64_t T, const clearmoe_router*
     a.dtype = rdtype;
     a.Wg = mlp ? mlp->W_out : router->W;
     a.bg = mlp ? mlp->b_out : router->b;
-    a.w_bf16 = mlp && L->desc.dtype == CLEARMOE_BF16;
+    a.w_bf16 = w_bf16;
     a.idx = L->idx;
     a.perm = L->perm;
     a.inv = L->inv;

@@ -39,9 +39,9 @@ __host__ __device__ inline int64_t n_class_tokens(int64_t T, int64_t cls_stride)
     return cls_stride > 0 ? (T + cls_stride - 1) / cls_stride : 0;
 }
 
-// Grid of the routing kernel for T tokens (one or two CTAs per SM); chunk = rows per CTA (a
-// routing range). Returns 0, -1 on a CUDA error, -2 when no launch shape fits.
-int route_grid(int64_t T, int d, int E, int dtype, int num_sms, int* grid, int* chunk);
+// Grid of the routing kernel for T tokens; chunk = rows per CTA (a routing range); w_bf16 as in RouteArgs.
+// Returns 0, -1 on a CUDA error, -2 when no launch shape fits.
+int route_grid(int64_t T, int d, int E, int dtype, int num_sms, int* grid, int* chunk, bool w_bf16 = false);
 int route_max_ctas(int num_sms, int dtype, int d, int E);
 // Phase 1 of the routing: idx, cta_counts and tinfo (no grid-wide step).
 cudaError_t launch_route(const RouteArgs& a, int grid, int chunk, cudaStream_t s);

@@ -299,7 +299,12 @@ __global__ void __launch_bounds__(RTC_THREADS, 1) route_tc_kernel(const __grid_c
 }
 
 // ------------------------------------------------------------------ fp32 router
-constexpr int RT_THREADS = 256;  // 8 warps
+// 8 warps for short ranges (two or more CTAs fit an SM, beside the next kernel's), 16 for longer ones (see
+// route_grid)
+constexpr int RT_ROWS_MIN = 16;
+constexpr int RT_THREADS = 256, RT_THREADS_LONG = 512;
+constexpr int rt_rows_short(bool w_bf16) { return w_bf16 ? 2 * RT_ROWS_MIN : RT_ROWS_MIN; }
+constexpr int rt_threads(int chunk, bool w_bf16) { return chunk > rt_rows_short(w_bf16) ? RT_THREADS_LONG : RT_THREADS; }
 constexpr size_t RT_F32_SMEM_MAX = 220 * 1024;
 
 // Dynamic shared memory: [W_g as fp32] [per-row word: expert | local rank << 8, when chunk words
@@ -318,8 +323,8 @@ __host__ __device__ inline RouteF32Layout route_f32_layout(int d, int E, int chu
     return L;
 }
 
-__global__ void __launch_bounds__(RT_THREADS) route_f32_kernel(const RouteArgs a, const int chunk) {
-    constexpr int NTHREADS = RT_THREADS;
+template <int NTHREADS>
+__global__ void __launch_bounds__(NTHREADS) route_f32_kernel(const RouteArgs a, const int chunk) {
     constexpr int NWARPS = NTHREADS / 32;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_count[CM_MAX_E];
@@ -550,23 +555,30 @@ __global__ void __launch_bounds__(256) route_finalize_kernel(const RouteArgs a, 
 // At most 32 rows of the histogram exchange per thread (a 32-bit mask of rows read).
 int route_max_ctas(int num_sms, int, int, int) { return min(num_sms * 8, 32 * RT_THREADS); }
 
-int route_grid(int64_t T, int d, int E, int dtype, int num_sms, int* grid, int* chunk) {
+int route_grid(int64_t T, int d, int E, int dtype, int num_sms, int* grid, int* chunk, bool w_bf16) {
     const bool bf16 = dtype == CLEARMOE_BF16;
     int occ = 0;
-    // bf16: one CTA per SM owns the ring. fp32: two per SM, but no more ranges than fc1's prefix table takes
-    // (256, and TC2_TAB_CAP entries of ranges x experts). The slots are then formed in fc1's epilogue, and the
-    // slot kernel, which the 304 ranges of two CTAs on every SM needed, is not launched: 5.3 us by itself;
-    // the DeiT-T layer at 12,608 tokens goes from 86 to 83.9 us.
+    // One CTA per SM: bf16's owns the ring, fp32's has 512 threads, as many as two of 256, in half the ranges.
+    // fc1's prefix table takes 256 ranges, and TC2_TAB_CAP entries of ranges x experts (152 at E = 16): within it
+    // the slots are formed in fc1's epilogue and the slot kernel (5.3 us by itself) is not launched. 256 threads
+    // in as many ranges as the table takes left SMs with half the warps: 50,432 fp32 tokens of d = 192 took
+    // (us, two CTAs of 256 on every SM / that / 512 threads) 25.4 / 31.7 / 22.0 with E = 4, 46.5 / 80.1 / 29.8 with
+    // E = 16, of d = 512 with E = 16 118 / 215 / 73. While ranges of 16 rows fit the table they go to CTAs of 256
+    // threads, beside which the next kernel's CTAs find room; for the MLP router of a bf16 layer, whose fc1 gains
+    // more by starting early, ranges of 32: ViT-B layer with 128 hidden units, 256 / 512 threads, 3,152 tokens 47.8 /
+    // 49.0 us, 8,000 78.0 / 80.1, 12,608 113 / 110; fp32 layers, 4,500 tokens of d = 192 47.2 / 46.5, 6,304 of
+    // d = 384 122 / 118.
     int64_t want = num_sms;
     if (!bf16) {
         const int64_t fit = TC2_TAB_CAP / (E > 0 ? E : 1) < 256 ? TC2_TAB_CAP / (E > 0 ? E : 1) : 256;
-        want = fit > num_sms ? (fit < 2 * num_sms ? fit : 2 * num_sms) : num_sms;
+        if (T <= fit * rt_rows_short(w_bf16)) want = fit;
     }
     // equal ranges over all CTAs (a range's last block may be partial)
     int64_t ch = (T + want - 1) / want;
     // the shared-memory attribute belongs to a device: set once per device
     if (smem_attr_once((const void*)route_tc_kernel, (int)RTC_SMEM_CAP) != cudaSuccess ||
-        smem_attr_once((const void*)route_f32_kernel, (int)RT_F32_SMEM_MAX) != cudaSuccess) {
+        smem_attr_once((const void*)route_f32_kernel<RT_THREADS>, (int)RT_F32_SMEM_MAX) != cudaSuccess ||
+        smem_attr_once((const void*)route_f32_kernel<RT_THREADS_LONG>, (int)RT_F32_SMEM_MAX) != cudaSuccess) {
         (void)cudaGetLastError();
         return -1;
     }
@@ -577,22 +589,24 @@ int route_grid(int64_t T, int d, int E, int dtype, int num_sms, int* grid, int* 
     }
     static std::mutex mu;
     std::lock_guard<std::mutex> lock(mu);
-    // occupancy queries are cached: (device, dtype, d, E, shared-memory bytes) -> CTAs per SM
-    static struct { int dev, dtype, d, E; size_t smem; int occ; } cache[64];
+    // occupancy queries are cached: (device, dtype, threads, d, E, shared-memory bytes) -> CTAs per SM
+    static struct { int dev, dtype, threads, d, E; size_t smem; int occ; } cache[64];
     static int ncache = 0;
     for (int iter = 0; iter < 4; ++iter) {
         const size_t smem = bf16 ? route_tc_layout(d).total : route_f32_layout(d, E, (int)ch).total;
+        const int threads = bf16 ? RTC_THREADS : rt_threads((int)ch, w_bf16);
         occ = -1;
         for (int i = 0; i < ncache; ++i)
-            if (cache[i].dev == dev && cache[i].dtype == dtype && cache[i].d == d && cache[i].E == E &&
-                cache[i].smem == smem)
+            if (cache[i].dev == dev && cache[i].dtype == dtype && cache[i].threads == threads && cache[i].d == d &&
+                cache[i].E == E && cache[i].smem == smem)
                 occ = cache[i].occ;
         if (occ < 0) {
-            const void* fn = bf16 ? (const void*)route_tc_kernel : (const void*)route_f32_kernel;
-            cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(
-                &occ, fn, bf16 ? RTC_THREADS : RT_THREADS, smem, cudaOccupancyDefault);
+            const void* fn = bf16 ? (const void*)route_tc_kernel
+                             : threads == RT_THREADS ? (const void*)route_f32_kernel<RT_THREADS>
+                                                     : (const void*)route_f32_kernel<RT_THREADS_LONG>;
+            cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(&occ, fn, threads, smem, cudaOccupancyDefault);
             if (err != cudaSuccess) return -1;
-            if (ncache < 64) cache[ncache++] = {dev, dtype, d, E, smem, occ};
+            if (ncache < 64) cache[ncache++] = {dev, dtype, threads, d, E, smem, occ};
         }
         if (occ <= 0) return -2;
         const int64_t maxg = (int64_t)occ * num_sms;
@@ -600,7 +614,7 @@ int route_grid(int64_t T, int d, int E, int dtype, int num_sms, int* grid, int* 
         want = maxg;
         ch = (T + want - 1) / want;
     }
-    if (ch < 16) ch = 16;
+    if (ch < RT_ROWS_MIN) ch = RT_ROWS_MIN;
     if (ch >= ((int64_t)1 << 24)) return -2;  // a row's local rank must fit in 24 bits
     *chunk = (int)ch;
     *grid = (int)((T + ch - 1) / ch);
@@ -618,9 +632,11 @@ cudaError_t launch_route(const RouteArgs& a, int grid, int chunk, cudaStream_t s
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (!bf16) {  // the attribute is set by route_grid
-        cfg.blockDim = dim3(RT_THREADS);
+        const int threads = rt_threads(chunk, a.w_bf16 != 0);
+        cfg.blockDim = dim3(threads);
         cfg.dynamicSmemBytes = route_f32_layout(a.d, a.E, chunk).total;
-        return cudaLaunchKernelEx(&cfg, route_f32_kernel, a, chunk);
+        return threads == RT_THREADS ? cudaLaunchKernelEx(&cfg, route_f32_kernel<RT_THREADS>, a, chunk)
+                                     : cudaLaunchKernelEx(&cfg, route_f32_kernel<RT_THREADS_LONG>, a, chunk);
     }
     if (a.d % RTC_BK != 0 || a.E > CM_MAX_E || a.T > ((int64_t)1 << 30)) return cudaErrorInvalidValue;
     RouteTcArgs t;

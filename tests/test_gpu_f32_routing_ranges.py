@@ -1,8 +1,9 @@
-"""The fp32 routing kernel takes as many ranges of tokens as fc1's prefix table holds (256, or 2,432 / E), so
-that fc1's epilogue forms the slots: expert counts on both sides of 2,432 / 256, one range more or less
-rows than a multiple. Routing against the
-oracle (bit-exact outside near ties; counts, offsets and perm the stable sort), outputs of sampled rows
-within the fp32 tolerance."""
+"""The fp32 routing kernel's ranges of tokens fit fc1's prefix table (256, or 2,432 / E), so that fc1's epilogue
+forms the slots: ranges of 16 rows in CTAs of 256 threads while they fit, then one range per SM in CTAs of 512.
+Token counts on both sides of that line for expert counts on both sides of 2,432 / 256, one row more or less
+than a multiple of the range. Routing against the oracle (bit-exact outside near ties; counts, offsets and
+perm the stable sort), outputs of sampled rows within the fp32 tolerance. And the time of routing does not grow
+with the number of experts as it did when sixteen experts left every SM half its warps."""
 import numpy as np
 import pytest
 import torch
@@ -22,7 +23,8 @@ def _built():
     assert torch.cuda.is_available(), "GPU tests need CUDA"
 
 
-@pytest.mark.parametrize("T,d,E", [(256 * 40, 192, 9), (256 * 40 + 1, 192, 10), (12608, 192, 4), (9001, 384, 16), (4097, 64, 1)])
+@pytest.mark.parametrize("T,d,E", [(256 * 40, 192, 9), (256 * 40 + 1, 192, 10), (12608, 192, 4), (9001, 384, 16), (4097, 64, 1),
+                                   (4096, 64, 4), (2432, 64, 16), (2433, 64, 16), (25216, 192, 8)])
 def test_ranges(T, d, E):
     L = synth.make_layer(synth.LayerShape("ranges", T, d, 4 * d, E, 16, "f32", n_cal=2000))
     D = synth.to_torch(L)
@@ -35,3 +37,29 @@ def test_ranges(T, d, E):
     y = oracle_rows(L, rows, gr["a"][rows])
     assert np.all(np.isfinite(out.float().cpu().numpy()))
     assert out_error(out[torch.from_numpy(rows).cuda()], y, "f32") <= tol("f32")
+
+
+def test_time_with_sixteen_experts():
+    g = torch.Generator(device="cuda").manual_seed(0)
+    T, d, t = 50432, 192, {}
+    x = torch.randn(T, d, generator=g, device="cuda")
+    h = cm.clearmoe_layer_create(T, d, 4 * d, 16, 16, cm.F32)
+    try:
+        for E in (4, 16):
+            W, b = torch.randn(E, d, generator=g, device="cuda"), torch.zeros(E, device="cuda")
+            runs = []
+            for _ in range(7):
+                a, z = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                cm.clearmoe_route(h, x, W, b)
+                torch.cuda.synchronize()
+                a.record()
+                for _ in range(20):
+                    cm.clearmoe_route(h, x, W, b)
+                z.record()
+                torch.cuda.synchronize()
+                runs.append(a.elapsed_time(z))
+            t[E] = sorted(runs)[3]
+        # the ratio was 1.8 with two CTAs of 256 threads on every SM, 2.5 with one, 1.35 with one of 512
+        assert t[16] < 2.1 * t[4], t
+    finally:
+        cm.clearmoe_layer_destroy(h)

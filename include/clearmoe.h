@@ -23,7 +23,7 @@
  *     and read the weights (every tensor argument except x), while the kernel enqueued just before it
  *     on the same stream is finishing; x is read only after that kernel has completed. So weights
  *     must not be written by the kernel immediately before the call (any later-enqueued work in
- *     between, or a synchronisation, is enough).
+ *     between, or a synchronisation, is enough). clearmoe_route_noalloc reads nothing early.
  *   - Arguments are validated on the host first; on a validation error (EINVAL, EUNSUPPORTED)
  *     nothing is enqueued and the outputs are untouched. CLEARMOE_ECUDA can also come from a
  *     launch after earlier kernels of the same call were enqueued; the outputs are then
@@ -324,6 +324,8 @@ int clearmoe_set_profile_events(clearmoe_layer* layer, void* const* events, int3
  *     must start at zero (the caller's status word; the histograms are rewritten before they are read).
  *     Calls whose work overlaps on the GPU (other streams, other host threads) race on the
  *     array: serialise them.
+ *   - Its first kernel may start while the kernel enqueued just before it on the same stream is
+ *     finishing, but reads nothing before that kernel has completed: x, W and b may be its output.
  *   - status (optional int32 device pointer, else NULL) is set to 0 at the start of the call and
  *     receives CLEARMOE_ETIMEOUT if a bounded device-side wait (1 s) runs out, in which case the
  *     outputs are undefined.

@@ -28,6 +28,7 @@ struct RouteArgs {
     // > 0: token t with t % cls_stride == 0 is a class token: it skips the router and forms group
     // E (idx = E), the dense path, whose slots follow every expert's: T - n_cls + t / cls_stride
     int64_t cls_stride;
+    int w_late;  // W_g may be the previous kernel's output: nothing is read before that kernel has completed
     int w_bf16;  // fp32 tokens (the MLP router's hidden layer) with bf16 W_g and b_g
     // x is the un-normalised stream y (nullable = x is the router's input as is): logits
     // rstd_t (W_g y_t - mean_t g) + b_g with (mean_t, rstd_t) = ln_stats[t], g_e = ln_wsum[e] = sum_k W_g[e, k]

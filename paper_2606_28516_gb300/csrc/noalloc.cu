@@ -104,6 +104,7 @@ extern "C" int clearmoe_route_noalloc(const void* x, int64_t T, int32_t d, int32
     a.dtype = dtype;
     a.Wg = router->W;
     a.bg = router->b;
+    a.w_late = 1;
     a.idx = idx;
     a.perm = perm;
     a.inv = nullptr;

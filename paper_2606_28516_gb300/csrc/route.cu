@@ -143,12 +143,17 @@ __global__ void __launch_bounds__(RTC_THREADS, 1) route_tc_kernel(const __grid_c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // W_g (a weight, not written by the previous kernel) is requested before the launch-overlap wait
-    if (producer && nblk > 0) {
-        mbar_arrive_expect_tx_warp(wbar, (uint32_t)(nk * RTC_WBOX_BYTES));
-        for (int kc = 0; kc < nk; ++kc) tma_load_2d(w_u32 + kc * RTC_WBOX_BYTES, &A.tmW, kc * RTC_BK, 0, wbar);
-    }
+    // W_g (a weight, not written by the previous kernel) is requested before the launch-overlap wait, or with
+    // w_late behind it
+    auto request_w = [&] {
+        if (producer && nblk > 0) {
+            mbar_arrive_expect_tx_warp(wbar, (uint32_t)(nk * RTC_WBOX_BYTES));
+            for (int kc = 0; kc < nk; ++kc) tma_load_2d(w_u32 + kc * RTC_WBOX_BYTES, &A.tmW, kc * RTC_BK, 0, wbar);
+        }
+    };
+    if (!a.w_late) request_w();
     pdl_wait();  // from here on the previous kernel's results (x) are read and outputs written
+    if (a.w_late) request_w();
     // the next kernel may start now (its CTAs set up, and may read x, while this one streams):
     // released only after the wait, so every kernel before this one has completed by then
     pdl_launch_dependents();
@@ -348,6 +353,7 @@ __global__ void __launch_bounds__(NTHREADS) route_f32_kernel(const RouteArgs a, 
 
     // ---------------- router logits + argmax for this CTA's rows
     float* Wf = reinterpret_cast<float*>(smem);
+    if (a.w_late) pdl_wait();
     if (a.w_bf16) {  // bf16 router weights on fp32 tokens: widened exactly
         const uint16_t* W = static_cast<const uint16_t*>(a.Wg);
         for (int i = tid; i < E * d; i += NTHREADS) Wf[i] = bf16_to_f32(W[i]);

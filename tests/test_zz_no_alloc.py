@@ -3,7 +3,8 @@
 device synchronisation): it keeps its scratch in a static device array instead of a handle's
 workspace. Checked through the C ABI against clearmoe_route, bit-exactly, on two calls in a row
 that reuse the same scratch (the second with a different token count and expert count), on the fp32
-routing kernel with and without a status word; tests/test_gpu_large_tokens.py runs it at 600,000
+routing kernel with and without a status word, and with router weights that the kernel enqueued just
+before writes; tests/test_gpu_large_tokens.py runs it at 600,000
 tokens, where the per-row words live in the caller's idx between the two kernels.
 This file is collected last on purpose, so a failure here leaves every other test already run."""
 import numpy as np
@@ -50,7 +51,7 @@ def test_route_noalloc_matches_route_twice():
 
 
 def test_route_noalloc_fp32_and_without_status_word():
-    """The fp32 routing kernel (two CTAs per SM, one token per lane) through the same entry point,
+    """The fp32 routing kernel through the same entry point,
     once with a status word and once without one (the array's spare word takes the status then),
     bit for bit against the handle's routing."""
     import __graft_entry__
@@ -66,6 +67,40 @@ def test_route_noalloc_fp32_and_without_status_word():
             assert int(status.item()) == 0
         for g, w, name in zip(got, want, ("idx", "counts", "offsets", "perm")):
             assert np.array_equal(g.cpu().numpy(), w), name
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_route_noalloc_reads_weights_written_just_before(dtype):
+    """W_g is the output of a dense FFN enqueued just before, whose last kernel lets its successor start early:
+    the routing follows the new weights, without a status word (no memset in between)."""
+    import __graft_entry__
+    __graft_entry__.build()
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(5)
+    w = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    T, d, H, E = 3000, 256, 4096, 8
+    x, bg = w(T, d).to(tdt), (0.1 * w(E)).to(tdt)
+    W1, b1, W2 = (0.06 * w(H, d)).to(tdt), (0.1 * w(H)).to(tdt), (0.05 * w(d, H)).to(tdt)
+    h = cm.clearmoe_layer_create(T, d, H, E, 16, cm.BF16 if dtype == "bf16" else cm.F32)
+    try:
+        src = [w(T, d).to(tdt) for _ in range(4)]
+        y, want = torch.empty(T, d, dtype=tdt, device="cuda"), []
+        for s in src:  # with a synchronisation in between
+            cm.clearmoe_dense_ffn_forward(h, s, W1, b1, W2, y)
+            torch.cuda.synchronize()
+            out = [torch.empty(n, dtype=torch.int32, device="cuda") for n in (T, E, E + 1, T)]
+            cm.clearmoe_route_noalloc(x, y[:E], bg, *out)
+            want.append(out)
+        assert not torch.equal(want[0][0], want[1][0])
+        for _ in range(20):
+            for s, ref in zip(src, want):
+                got = [torch.empty(n, dtype=torch.int32, device="cuda") for n in (T, E, E + 1, T)]
+                cm.clearmoe_dense_ffn_forward(h, s, W1, b1, W2, y)
+                cm.clearmoe_route_noalloc(x, y[:E], bg, *got)
+                for a, b in zip(got, ref):
+                    assert torch.equal(a, b)
+    finally:
+        cm.clearmoe_layer_destroy(h)
 
 
 def test_route_noalloc_rejects_bad_sizes():

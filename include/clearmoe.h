@@ -291,12 +291,13 @@ int clearmoe_get_routing(clearmoe_layer* layer, int32_t* idx, int32_t* counts, i
  * part-counted, so that the next calls run on a consistent handle. */
 int clearmoe_layer_status(clearmoe_layer* layer);
 
-/* Fault injection for tests of the bounded waits: every device-side wait of the routing kernel
- * gives up after wait_limit_ns nanoseconds (default 1e9) and, when phantom_arrivals > 0, the
+/* Fault injection for tests of the bounded waits: every device-side wait of the handle's kernels
+ * gives up after wait_limit_ns nanoseconds (default 1e9, at least 1,000; the hardware may suspend a
+ * wait for some microseconds before the limit is looked at) and, when phantom_arrivals > 0, the
  * bf16 routing withholds the copy of its first stage (the first K blocks of its first 128-row block,
- * in its first CTA), so the MMA thread's wait for it runs out and the call reports
- * CLEARMOE_ETIMEOUT through clearmoe_layer_status; the kernel lets its other copies in flight land
- * before it exits, and the layer stays usable. phantom_arrivals = 0 restores normal use. */
+ * in its first CTA), so that the MMA warp's wait for it runs out and the call reports
+ * CLEARMOE_ETIMEOUT through clearmoe_layer_status. A kernel that gave up lets its copies in flight
+ * land before it exits, and the layer stays usable. phantom_arrivals = 0 restores normal use. */
 int clearmoe_debug_set_wait(clearmoe_layer* layer, int64_t wait_limit_ns, int32_t phantom_arrivals);
 
 /* Per-stage timing: when n >= 5, clearmoe_ffn_forward records events[0] before its first kernel

@@ -61,7 +61,6 @@ int cuda_fail(cudaError_t e) {
     return CLEARMOE_ECUDA;
 }
 
-// The fp32 layers' SIMT GEMMs, with the handle's split-K workspace.
 // The fp32 tensor-core GEMMs' tiling: N tile and K split for an [M x N] x K product (row tiles:
 // ceil(M / 128) + extra), with the handle's split workspace and counters (fp32 layers own them).
 cm::TcTf32Plan tf32_plan(const clearmoe_layer* L, cm::TcGemmArgs& g, int N, int K, int64_t M, int extra_tiles) {
@@ -77,6 +76,7 @@ cm::TcTf32Plan tf32_plan(const clearmoe_layer* L, cm::TcGemmArgs& g, int N, int 
     return p;
 }
 
+// The fp32 layers' SIMT GEMMs, with the handle's split-K workspace.
 int launch_simt(clearmoe_layer* L, cm::SimtGemmArgs& g, cudaStream_t s) {
     g.ws = L->simt_ws;
     g.ws_floats = L->simt_ws ? cm::simt_ws_floats(L->num_sms) : 0;

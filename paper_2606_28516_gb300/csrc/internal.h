@@ -154,7 +154,7 @@ struct TcGemmArgs {
     int64_t ldc;
     int32_t* status;
     int64_t wait_limit_ns;
-    // 2-SM dense kernel only: output row m (a token) goes to its routing slot offsets[e] +
+    // dense mode of the 2-SM and fp32 kernels: output row m (a token) goes to its routing slot offsets[e] +
     // (tokens of e in ranges before m's) + rank, with (e, rank) = rt_info[m] packed as e | rank << 8
     // and m's range m / rt_chunk; the kernel forms the prefix table from rt_counts ([rt_ctas x
     // CM_MAX_E], rt_ctas <= 256, rt_ctas * rt_E <= TC2_TAB_CAP) and writes perm, counts, offsets.

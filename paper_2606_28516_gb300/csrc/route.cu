@@ -7,8 +7,8 @@
 // range's earlier tokens of that expert << 8) to tinfo. The slot of token t in range c is
 // offsets[e] + (tokens of e in ranges before c) + its rank, in token order within each expert,
 // which makes the sort stable. It is formed by the consumer of the routing: the fc1 epilogue of
-// the 2-SM GEMM (which then stores z rows at their slots and writes perm), or route_finalize_kernel
-// (perm and inv ahead of the other paths).
+// the 2-SM and fp32 GEMMs (which then store z rows at their slots and write perm), or
+// route_finalize_kernel (perm and inv ahead of the other paths).
 //
 // bf16 tokens (route_tc_kernel): the d x E contraction runs on the tensor cores. One CTA per SM
 //   streams its range as 128-row blocks into a ring of shared-memory stages, each stage nkc K blocks

@@ -38,7 +38,8 @@
 // Measured (DeiT-T layer, whole forwards): T = 12,608: 125 us with both operands in shared memory, 112
 // with coalesced stores, 93 with A in tensor memory, 87.5 with the branch-free GELU, 86 with no option tests,
 // 83.9 without the slot kernel (route_grid), 79.5 with the products started beside the previous kernel, 77.0
-// with whole warps staging their rows; T = 788: 48.1 / 42.5 / 38.8 / 37.1 / 34.6 / 34.0 / 30.4 / 30.4 us.
+// with whole warps staging their rows, 75.7 with the routing on 512 threads a CTA; T = 788: 48.1 / 42.5 / 38.8 /
+// 37.1 / 34.6 / 34.0 / 30.4 / 30.4 / 30.6 us.
 #include <cstdint>
 #include <mutex>
 

@@ -16,7 +16,8 @@
 // the last group is the class tokens' dense path, K chain z x W2 alone). Store epilogues may add
 // an output bias (fc2's b2). With a.rows set,
 // output row m goes to C[a.rows[m]] (fc1: inv[token] = slot; grouped: perm[slot] = token).
-// Every wait is bounded; both CTAs always reach the closing cluster barrier.
+// Every wait is bounded; both CTAs always reach the closing cluster barrier, and the issuer of a CTA that
+// gave up waits before it for the copies still in flight.
 #include "common.cuh"
 #include "drain.h"
 #include "internal.h"

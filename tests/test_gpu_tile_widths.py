@@ -1,5 +1,5 @@
-"""The 2-SM kernels' tile width follows the token count (fc1: 256 or 128 columns by rounds of
-tiles; experts and dense fc2: the narrowest tile that runs in one round). Every width sums each output over K in the same
+"""The 2-SM kernels' tile width follows the token count (fc1: 256 or 128 columns by rounds of tiles; experts and
+dense fc2: the narrowest tile that runs in one round). Every width sums each output over K in the same
 order, so a batch cut into pieces that take other widths gives the same bits: sizes on both sides of
 each line, ragged last blocks, one expert and several, both basis forms and the dense FFN."""
 import pytest

@@ -56,7 +56,10 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // in GELU (8.3e-8). Past 5.5 it falls on until t = 14, where t is held and the second term is 2e-35.
 // Horner's rule runs on v = -t with the odd coefficients' signs turned, and the factor 1/2 is a -1 in the
 // exponent, so that the result is one fma: 7 packed fp32x2 operations and two ex2 a pair, and one more for
-// the infinities. What it costs is fc1's bound in short K and its energy in long.
+// the infinities. What it costs is fc1's bound in short K and its energy in long: with the rational form named
+// below (12 packed operations, two reciprocals) the ViT-B layer at 50,432 tokens took 400 us under load, now
+// 390, the dense FFN at 100,864 tokens 652 and 634, the 12-sublayer stack at 25,216 tokens 2,385 and 2,348, the
+// DeiT-S layer at 12,608 tokens 48.8 and 48.5.
 // Error against float64: at most 3.2e-7 for every u (the rational form of Abramowitz & Stegun 7.1.28 in fp32:
 // 7.1e-7), in every interval below -5 smaller than that form's, and mean square below it at every width
 // (tests/test_gelu_exp2.py). These are absolute bounds: down to u = -4.25 the error is at most a quarter of the

@@ -22,7 +22,7 @@ struct TmapKey {
 // Replacement in order misses every lookup of a program that cycles through more keys than fit, and a call
 // encodes up to 40 (a layer of E = 16 experts: 16 expert matrices and three others, each also in boxes of
 // half the rows, and x, z, t, W_g): 2,048 hold a model of 24 such layers with room for other token counts. 64
-// held 12 sublayers of E = 8 at a third of its lookups. A miss is a driver call; a hit costs the lock, one or two
+// held 12 sublayers of E = 8 at a third of its lookups. A miss is a call into the CUDA driver; a hit costs the lock, one or two
 // comparisons and a copy of 128 bytes. Zero-initialised storage is an empty cache.
 template <class Map, int CAP = 2048>
 class TmapCache {
